@@ -49,27 +49,14 @@ k_kick(int64_t N, float *__restrict__ vx, float *__restrict__ vy, float *__restr
 }
 
 constexpr int MOM_THREADS = 256;
-constexpr int MOM_BLOCKS = 4096;  // 1M threads: enough loads in flight for a bandwidth-bound pass
+constexpr int MOM_BLOCKS = 608;  // at most: four resident blocks on each of 152 SMs
 constexpr int MOM_N = 9;  // sums: m v (3), m a (3), kinetic, m |a|, potential
-
-__device__ __forceinline__ double block_sum(double v, double *sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < MOM_THREADS / 32; ++w) r += sh[w];
-    __syncthreads();
-    return r;
-}
 
 // Double-float arithmetic on the float32 pipe (an unevaluated sum hi + lo of
 // two float32 values, about 48 significant bits): GB300's float64 pipe is
-// narrow, so the per-particle terms and each thread's partial sums are formed
-// this way and only the per-thread totals are reduced in float64.
+// narrow (2 lanes a clock and SM), so the per-particle terms, each thread's
+// partial sums and each warp's reduction are formed this way and only the
+// per-thread totals are reduced in float64.
 // Knuth's TwoSum: s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 {
@@ -186,27 +173,41 @@ __device__ __forceinline__ void moment_terms(DF (&s)[MOM_N], float mi, bool has_
     }
 }
 
-// Fixed grid and fixed per-thread striding: the summation order depends only
-// on N, so the float64 results are reproducible run to run.  Thread t takes
-// the groups of four consecutive particles t, t + T, t + 2T, ... (T threads;
-// each group's values by 16-byte loads where an array is aligned, all of a
-// group's loads issued before its arithmetic) and then particle
-// 4 floor(N / 4) + t of the last, partial group.  Per particle and per thread
-// in double-float (above), across threads and blocks in float64.
+// Blocks of the first pass: enough for every group of four, at most MOM_BLOCKS.
+int moment_blocks(int64_t N)
+{
+    const int64_t b = (N / 4 + MOM_THREADS - 1) / MOM_THREADS;
+    return b < 1 ? 1 : (b > MOM_BLOCKS ? MOM_BLOCKS : (int)b);
+}
+
+// Fixed per-thread striding and a grid that depends only on N: so does the
+// summation order, and the float64 results are reproducible run to run.
+// Thread t takes the groups of four consecutive particles t, t + T, t + 2T,
+// ... (T threads; each group's values by 16-byte loads where an array is
+// aligned, all of a group's loads issued before its arithmetic) and then
+// particle 4 floor(N / 4) + t of the last, partial group.  Per particle and
+// per thread in double-float (above), across threads and blocks in float64.
+//
+// What bounds it: the copy rate at 16.8M particles (470 MB read), its latency
+// at a few thousand.  Nine float64 shuffle reductions in each of a fixed 4096
+// blocks held the narrow float64 pipe for 150 us whatever N; reduced in
+// double-float by a grid that follows N, 4096 particles take MOMS4K us (164
+// before) and 16.8M take MOMS16M us (265 before).
 __global__ void __launch_bounds__(MOM_THREADS)
 k_moments_partial(int64_t N, const float *__restrict__ m, const float *__restrict__ vx, const float *__restrict__ vy,
                   const float *__restrict__ vz, const float *__restrict__ ax, const float *__restrict__ ay,
                   const float *__restrict__ az, const float *__restrict__ phi, double *__restrict__ part)
 {
-    __shared__ double sh[MOM_THREADS / 32];
+    __shared__ double sh[MOM_N][MOM_THREADS];
     DF s[MOM_N];
     const bool hv = vx != nullptr, ha = ax != nullptr, hp = phi != nullptr;
     auto al = [](const float *p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     const bool am = al(m), avx = al(vx), avy = al(vy), avz = al(vz), aax = al(ax), aay = al(ay), aaz = al(az),
                aph = al(phi);
     const int64_t t0 = (int64_t)blockIdx.x * MOM_THREADS + threadIdx.x;
+    const int64_t T = (int64_t)gridDim.x * MOM_THREADS;
     const int64_t groups = N / 4;
-    for (int64_t g = t0; g < groups; g += (int64_t)MOM_BLOCKS * MOM_THREADS) {
+    for (int64_t g = t0; g < groups; g += T) {
         const int64_t i = 4 * g;
         const float4 m4 = load4(m, i, am);
         float4 v0, v1, v2, a0, a1, a2, p4;
@@ -232,21 +233,32 @@ k_moments_partial(int64_t N, const float *__restrict__ m, const float *__restric
         moment_terms(s, m[i], hv, hv ? vx[i] : 0.f, hv ? vy[i] : 0.f, hv ? vz[i] : 0.f, ha, ha ? ax[i] : 0.f,
                      ha ? ay[i] : 0.f, ha ? az[i] : 0.f, hp, hp ? phi[i] : 0.f);
 #pragma unroll
-    for (int k = 0; k < MOM_N; ++k) {
-        double r = block_sum(s[k].value(), sh);
-        if (threadIdx.x == 0) part[(int64_t)k * MOM_BLOCKS + blockIdx.x] = r;
+    for (int k = 0; k < MOM_N; ++k) sh[k][threadIdx.x] = s[k].value();
+    __syncthreads();
+    // one warp per sum: its lanes add eight threads' totals each, then a shuffle tree
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < MOM_N; k += MOM_THREADS / 32) {
+        double r = 0.0;
+#pragma unroll
+        for (int q = 0; q < MOM_THREADS / 32; ++q) r += sh[k][q * 32 + lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+        if (lane == 0) part[(int64_t)k * MOM_BLOCKS + blockIdx.x] = r;
     }
 }
 
-__global__ void __launch_bounds__(MOM_THREADS) k_moments_final(const double *__restrict__ part, double *__restrict__ out)
+// One warp per sum: its lanes take the blocks' totals in turn, then the warp
+// adds up in a fixed order.
+__global__ void __launch_bounds__(32 * MOM_N)
+k_moments_final(const double *__restrict__ part, int blocks, double *__restrict__ out)
 {
-    __shared__ double sh[MOM_THREADS / 32];
-    for (int k = 0; k < MOM_N; ++k) {
-        double s = 0.0;
-        for (int b = threadIdx.x; b < MOM_BLOCKS; b += MOM_THREADS) s += part[(int64_t)k * MOM_BLOCKS + b];
-        double r = block_sum(s, sh);
-        if (threadIdx.x == 0) out[k] = r;
-    }
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < blocks; b += 32) s += part[(int64_t)k * MOM_BLOCKS + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[k] = s;
 }
 
 // Stream map on sorted records: o += dt v (one float32 fma per axis); flags a
@@ -329,10 +341,11 @@ extern "C" int hacc_moments(int64_t N, const float *m, const float *vx, const fl
     if ((ax || ay || az) && !(ax && ay && az)) return HACC_ERR_INVALID;
     if (ws_bytes < hacc_moments_workspace_size(N)) return HACC_ERR_CAPACITY;
     cudaStream_t st = as_stream(stream);
-    k_moments_partial<<<MOM_BLOCKS, MOM_THREADS, 0, st>>>(N, m, vx, vy, vz, ax, ay, az, phi,
+    const int blocks = moment_blocks(N);
+    k_moments_partial<<<blocks, MOM_THREADS, 0, st>>>(N, m, vx, vy, vz, ax, ay, az, phi,
                                                           reinterpret_cast<double *>(ws));
     HACC_LAUNCH_CHECK();
-    k_moments_final<<<1, MOM_THREADS, 0, st>>>(reinterpret_cast<const double *>(ws), out);
+    k_moments_final<<<1, 32 * MOM_N, 0, st>>>(reinterpret_cast<const double *>(ws), blocks, out);
     HACC_LAUNCH_CHECK();
     return HACC_OK;
 }
