@@ -146,17 +146,13 @@ __device__ __forceinline__ void tile_potential(const float4 *__restrict__ tj, in
     }
 }
 
-// Adjoint pair loop over one staged tile.  Per pair, with f = f_SR(s) and
-// fp2 = 2 f_SR'(s):  U += f lam_j ;  V += m_j f ;
-// X += fp2 (m_i (d.lam_j) - m_j (d.lam_i)) d ;  G += f (d.lam_j).
-// Then dL/dx_i = m_i U - lam_i V + X and dL/dm_i = -G.
-// Equal masses (EQ): V += f and X += fp2 (d.(lam_j - lam_i)) d, so that
-// dL/dx_i = m (U - lam_i V + X).
-// Without G (the W form) the three sums fold into one: with mu = m_i lam_j -
-// m_j lam_i, W += f mu + fp2 (d.mu) d and dL/dx_i = W (equal masses: mu / m
-// summed, dL/dx_i = m W).
-// One pair of the adjoint, accumulated into acc[8] = (U, V, X, G) of one i
-// (the W form: acc[3] = W).
+// One pair of the adjoint, accumulated into acc = (W, G) of one i: with f =
+// f_SR(s), fp2 = 2 f_SR'(s) and mu = m_i lam_j - m_j lam_i (equal masses, EQ:
+// mu / m = lam_j - lam_i),
+//   W += f mu + fp2 (d.mu) d      dL/dx_i = W (equal masses: m W)
+//   G += f (d.lam_j)              dL/dm_i = -G (GM only)
+// Summing the antisymmetric pair term takes the cancellation between the lam_j
+// and lam_i parts of a close pair out of the totals.
 template <bool GM, bool EQ>
 __device__ __forceinline__ void pair_adjoint(const float4 p, const float4 l, float oxp, float oyp, float ozp,
                                              float mi, float lix, float liy, float liz, const PairConsts &K,
@@ -172,45 +168,35 @@ __device__ __forceinline__ void pair_adjoint(const float4 p, const float4 l, flo
     float f = t3 + q;
     float qp = fmaf(fmaf(fmaf(fmaf(K.kp[4], se, K.kp[3]), se, K.kp[2]), se, K.kp[1]), se, K.kp[0]);
     float fp2 = fmaf(-3.0f, t3 * t2, qp);
-    if constexpr (!GM) {
-        float ex, ey, ez;  // mu (equal masses: mu / m)
-        if constexpr (EQ) {
-            ex = l.x - lix;
-            ey = l.y - liy;
-            ez = l.z - liz;
-        } else {
-            ex = fmaf(mi, l.x, -(p.w * lix));
-            ey = fmaf(mi, l.y, -(p.w * liy));
-            ez = fmaf(mi, l.z, -(p.w * liz));
-        }
-        const float r = fp2 * fmaf(dz, ez, fmaf(dy, ey, dx * ex));
+    float ex, ey, ez;  // mu (equal masses: mu / m)
+    if constexpr (EQ) {
+        ex = l.x - lix;
+        ey = l.y - liy;
+        ez = l.z - liz;
+    } else {
+        ex = fmaf(mi, l.x, -(p.w * lix));
+        ey = fmaf(mi, l.y, -(p.w * liy));
+        ez = fmaf(mi, l.z, -(p.w * liz));
+    }
+    const float r = fp2 * fmaf(dz, ez, fmaf(dy, ey, dx * ex));
+    // the accumulations of this pair happen only inside the cutoff
+    if constexpr (GM) {
+        const float dlj = fmaf(dz, l.z, fmaf(dy, l.y, dx * l.x));
+        asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %4, %5;\n\t"
+            "@p fma.rn.f32 %0, %6, %7, %0;\n\t@p fma.rn.f32 %1, %6, %8, %1;\n\t@p fma.rn.f32 %2, %6, %9, %2;\n\t"
+            "@p fma.rn.f32 %0, %10, %11, %0;\n\t@p fma.rn.f32 %1, %10, %12, %1;\n\t"
+            "@p fma.rn.f32 %2, %10, %13, %2;\n\t@p fma.rn.f32 %3, %6, %14, %3;\n\t}"
+            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
+            : "f"(se), "f"(K.rc2e), "f"(f), "f"(ex), "f"(ey), "f"(ez), "f"(r), "f"(dx), "f"(dy), "f"(dz), "f"(dlj));
+    } else {
         asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %3, %4;\n\t"
             "@p fma.rn.f32 %0, %5, %6, %0;\n\t@p fma.rn.f32 %1, %5, %7, %1;\n\t@p fma.rn.f32 %2, %5, %8, %2;\n\t"
             "@p fma.rn.f32 %0, %9, %10, %0;\n\t@p fma.rn.f32 %1, %9, %11, %1;\n\t@p fma.rn.f32 %2, %9, %12, %2;\n\t}"
             : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2])
             : "f"(se), "f"(K.rc2e), "f"(f), "f"(ex), "f"(ey), "f"(ez), "f"(r), "f"(dx), "f"(dy), "f"(dz));
-        return;
     }
-    float dlj = fmaf(dz, l.z, fmaf(dy, l.y, dx * l.x));
-    float r;
-    if constexpr (EQ) {
-        r = fp2 * (dlj - fmaf(dz, liz, fmaf(dy, liy, dx * lix)));
-    } else {
-        const float dli = fmaf(dz, liz, fmaf(dy, liy, dx * lix));
-        r = fp2 * fmaf(mi, dlj, -(p.w * dli));
-    }
-    const float mj = EQ ? 1.0f : p.w;
-    // the accumulations of this pair happen only inside the cutoff
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %8, %9;\n\t"
-        "@p fma.rn.f32 %0, %10, %11, %0;\n\t@p fma.rn.f32 %1, %10, %12, %1;\n\t@p fma.rn.f32 %2, %10, %13, %2;\n\t"
-        "@p fma.rn.f32 %3, %14, %10, %3;\n\t"
-        "@p fma.rn.f32 %4, %15, %16, %4;\n\t@p fma.rn.f32 %5, %15, %17, %5;\n\t@p fma.rn.f32 %6, %15, %18, %6;\n\t"
-        "@p fma.rn.f32 %7, %10, %19, %7;\n\t}"
-        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]), "+f"(acc[4]), "+f"(acc[5]), "+f"(acc[6]),
-          "+f"(acc[7])
-        : "f"(se), "f"(K.rc2e), "f"(f), "f"(l.x), "f"(l.y), "f"(l.z), "f"(mj), "f"(r), "f"(dx), "f"(dy),
-          "f"(dz), "f"(dlj));
 }
+
 
 // Adjoint pair loop over one staged tile (positions tj, cotangents tl).
 template <int MODE, int IPL, bool EQ>
@@ -410,25 +396,13 @@ __device__ __forceinline__ bool run_task(const KArgs &a, Ring<MODE, JT, STAGES> 
             // the sum met particle i itself once (d = 0, se = eps exactly): take that term out
             const float self = pair_potential_of(K.eps, K);
             a.out_x[o] = (A.h[u][0] + A.l[u][0]) - oi[u].w * self;
-        } else if constexpr (adj_wform(MODE)) {
-            // dL/dx_i = W (equal masses: m W)
+        } else {
+            // dL/dx_i = W (equal masses: m W) ;  dL/dm_i = -G
             const float sc = EQ ? oi[u].w : 1.0f;
             a.out_x[o] = sc * A.total(u, 0);
             a.out_y[o] = sc * A.total(u, 1);
             a.out_z[o] = sc * A.total(u, 2);
-        } else {
-            // dL/dx_i = m_i U - lam_i V + X (equal masses: m (U - lam_i V + X)) ;  dL/dm_i = -G
-            const float Vs = A.total(u, 3);
-            if constexpr (EQ) {
-                a.out_x[o] = oi[u].w * (A.total(u, 0) + fmaf(-li[u].x, Vs, A.total(u, 4)));
-                a.out_y[o] = oi[u].w * (A.total(u, 1) + fmaf(-li[u].y, Vs, A.total(u, 5)));
-                a.out_z[o] = oi[u].w * (A.total(u, 2) + fmaf(-li[u].z, Vs, A.total(u, 6)));
-            } else {
-                a.out_x[o] = fmaf(oi[u].w, A.total(u, 0), fmaf(-li[u].x, Vs, A.total(u, 4)));
-                a.out_y[o] = fmaf(oi[u].w, A.total(u, 1), fmaf(-li[u].y, Vs, A.total(u, 5)));
-                a.out_z[o] = fmaf(oi[u].w, A.total(u, 2), fmaf(-li[u].z, Vs, A.total(u, 6)));
-            }
-            if constexpr (MODE == ADJOINT_GM) a.out_m[o] = -A.total(u, 7);
+            if constexpr (MODE == ADJOINT_GM) a.out_m[o] = -A.total(u, 3);
         }
     }
     return true;
@@ -436,7 +410,7 @@ __device__ __forceinline__ bool run_task(const KArgs &a, Ring<MODE, JT, STAGES> 
 
 // Persistent work-stealing kernel: each warp takes tasks from a global
 // counter until none is left.  A task of more than 32 particles runs two i
-// particles per lane (four, above 64, in the adjoint's W form), one of at most
+// particles per lane (four, above 64, in the adjoint), one of at most
 // 16 runs each i on two lanes.
 // Register budgets: the forward and potential kernels keep 80 registers so that
 // 3 CTAs (24 warps) fit an SM; the adjoint's staging needs twice the shared
@@ -481,9 +455,8 @@ __global__ void __launch_bounds__(256, min_ctas(MODE)) k_pairs(const KArgs a)
         if (!take_task(a, t, lane, task, a.order)) continue;
         const hacc_volume &vol = a.vols[task.w];
         bool ok = true;
-        // sub-chunks of larger tasks: 128 particles (four i per lane) for the adjoint's W form,
-        // whose three sums leave the registers for it, else 64
-        constexpr int CHUNK = adj_wform(MODE) ? 128 : 64;
+        // sub-chunks of larger tasks: 128 particles (four i per lane) for the adjoint, else 64
+        constexpr int CHUNK = is_adjoint(MODE) ? 128 : 64;
         for (int sb = task.y; ok && sb < task.z; sb += CHUNK) {
             const int se = min(sb + CHUNK, task.z);
             if (CHUNK == 128 && se - sb > 64)

@@ -191,22 +191,18 @@ __device__ __forceinline__ float rsqrt_hw(float x)
     return y;
 }
 
-// Adjoint accumulator layout (sizes the adjoint's shared memory): room for
-// two i per lane with eight sums each (four i with the W form's three fit).
-constexpr int ADJ_NACC = 8;
-constexpr int ADJ_IPL_MAX = 2;
+// Adjoint sums per i particle (the W form): with mu = m_i lam_j - m_j lam_i,
+// W (3) = sum f mu + fp2 (d.mu) d = dL/dx_i (equal masses: mu / m summed,
+// dL/dx_i = m W), and with dL/dm G = sum f d.lam_j = -dL/dm_i.  Float32 partial
+// sums live in registers for one tile; the compensated (hi, lo) totals live in
+// shared memory, lane-contiguous, room for four i per lane, so that they fit
+// the register budget.  Four sums with dL/dm where the factored form (U, V, X,
+// G) took eight: the symmetric adjoint with dL/dm went from 2.90 to 2.59 ms on
+// 2.1M lattice particles and from 21.1 to 20.2 ms on 4.1M clustered ones.
+constexpr int ADJ_NACC = 4;
+constexpr int ADJ_IPL_MAX = 4;
 constexpr int ADJ_COMP_BYTES = ADJ_IPL_MAX * ADJ_NACC * 2 * 32 * 4;
-
-// Adjoint accumulators per i particle: U (3) = sum f lam_j, V = sum m_j f,
-// X (3) = sum fp2 (m_i d.lam_j - m_j d.lam_i) d, G = sum f d.lam_j (with dL/dm
-// only).  Without dL/dm (the W form) the three sums collapse into one
-// vector: with mu = m_i lam_j - m_j lam_i, W (3) = sum f mu + fp2 (d.mu) d =
-// dL/dx_i (equal masses: mu / m summed, dL/dx_i = m W).  Float32 partial sums
-// live in registers for one tile; the compensated (hi, lo) totals live in
-// shared memory, lane-contiguous, so that two i particles per lane fit the
-// register budget.
-__host__ __device__ constexpr bool adj_wform(int mode) { return mode == ADJOINT; }
-__host__ __device__ constexpr int adj_nacc(int mode) { return mode == ADJOINT_GM ? 8 : (adj_wform(mode) ? 3 : 7); }
+__host__ __device__ constexpr int adj_nacc(int mode) { return mode == ADJOINT_GM ? 4 : 3; }
 
 template <int MODE, int IPL, int NC = adj_nacc(MODE)>
 struct AccAdj {
@@ -372,8 +368,8 @@ void pair_consts(const hacc_sr_params *p, PairConsts &K)
 
 // Workspace of the pair calls: the task counter, the adjoints' sorted
 // cotangents (16 B per particle), and the symmetric kernels' float64 sums
-// (3 per particle for the force, 8 for the adjoint).
-constexpr int SYM_ACC_MAX = 8;
+// (3 per particle for the force, 3 or 4 for the adjoint).
+constexpr int SYM_ACC_MAX = 4;
 
 struct ForceWs {
     int32_t *counter;

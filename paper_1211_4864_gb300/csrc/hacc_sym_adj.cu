@@ -11,30 +11,24 @@ namespace {
 // Symmetric adjoint.  The pair (i, j)'s terms of the vector-Jacobian product
 // are antisymmetric in dL/dx (J(d) = f I + 2 f' d d^T is even in d):
 //   dL/dx_i += m_i J lam_j - m_j J lam_i,   dL/dx_j gets the same with minus,
-// so each pair is evaluated once.  Both sides keep the gather adjoint's
-// factored sums, U = sum f lam_p, V = sum m_p f, X = sum r d_k (r = 2 f'
-// (m_k d_k.lam_p - m_p d_k.lam_k)), G = sum f d_k.lam_p, over partners p with
-// d_k = x_p - x_k, so that dL/dx_k = m_k U - lam_k V + X and dL/dm_k = -G.
-// For the pair seen from j every term flips sign or swaps: U_j += f lam_i,
-// V_j += m_i f, X_j -= r d, G_j -= f d.lam_i.
-// Without dL/dm (the W form): with mu = m_i lam_j - m_j lam_i the pair's
-// whole term w = f mu + fp2 (d.mu) d is antisymmetric, like a force, so i
-// adds w and j subtracts it; each side carries three sums (u0, u1, u2) and
-// dL/dx_k = W_k (equal masses: mu / m summed, dL/dx_k = m W_k).
+// so each pair is evaluated once.  With mu = m_i lam_j - m_j lam_i the pair's
+// whole term w = f mu + fp2 (d.mu) d (fp2 = 2 f') is antisymmetric, like a
+// force: i adds w and j subtracts it, three sums W per particle, dL/dx_k = W_k
+// (equal masses: mu / m summed, dL/dx_k = m W_k).  With dL/dm a fourth, G: i
+// adds f d.lam_j and j subtracts f d.lam_i, dL/dm_k = -G_k.
 // ---------------------------------------------------------------------------
 
 // One j of an adjoint rotation block: record shifted into the i frame, its
 // cotangent, its partial sums and sorted slot (-1: empty lane).
 struct JAdj {
     float x, y, z, m, lx, ly, lz;
-    float u0, u1, u2, v, x0, x1, x2, g;
+    float w0, w1, w2, g;
     int slot;
 };
 
 template <bool GM, bool EQ>
 __device__ __forceinline__ void rotate_adj(JAdj &J, int src)
 {
-    constexpr bool WF = adj_wform(GM ? ADJOINT_GM : ADJOINT);
     J.x = __shfl_sync(FULL, J.x, src);
     J.y = __shfl_sync(FULL, J.y, src);
     J.z = __shfl_sync(FULL, J.z, src);
@@ -42,21 +36,15 @@ __device__ __forceinline__ void rotate_adj(JAdj &J, int src)
     J.lx = __shfl_sync(FULL, J.lx, src);
     J.ly = __shfl_sync(FULL, J.ly, src);
     J.lz = __shfl_sync(FULL, J.lz, src);
-    J.u0 = __shfl_sync(FULL, J.u0, src);
-    J.u1 = __shfl_sync(FULL, J.u1, src);
-    J.u2 = __shfl_sync(FULL, J.u2, src);
-    if constexpr (WF) return;
-    J.v = __shfl_sync(FULL, J.v, src);
-    J.x0 = __shfl_sync(FULL, J.x0, src);
-    J.x1 = __shfl_sync(FULL, J.x1, src);
-    J.x2 = __shfl_sync(FULL, J.x2, src);
+    J.w0 = __shfl_sync(FULL, J.w0, src);
+    J.w1 = __shfl_sync(FULL, J.w1, src);
+    J.w2 = __shfl_sync(FULL, J.w2, src);
     if constexpr (GM) J.g = __shfl_sync(FULL, J.g, src);
 }
 
 // One pair of the adjoint, both sides; outside the cutoff (or outside the
 // upper triangle of a diagonal block) f and r are zero, so every sum is
-// unchanged.  Equal masses (EQ): V sums f on both sides and r = fp2
-// d.(lam_j - lam_i) (the W form: mu / m), the common mass applied by the
+// unchanged.  Equal masses (EQ): mu / m, the common mass applied by the
 // finishing pass.
 template <bool GM, bool EQ>
 __device__ __forceinline__ void pair_adj_sym(JAdj &J, const float4 &oi, const float4 &li, const PairConsts &K,
@@ -73,54 +61,28 @@ __device__ __forceinline__ void pair_adj_sym(JAdj &J, const float4 &oi, const fl
     const float fp2 = fmaf(-3.0f, t3 * t2, qp);
     const bool in = ok & (se < K.rc2e);
     const float f = in ? t3 + q : 0.0f;
-    if constexpr (!GM) {  // the W form
-        float ex, ey, ez;  // mu (equal masses: mu / m)
-        if constexpr (EQ) {
-            ex = J.lx - li.x;
-            ey = J.ly - li.y;
-            ez = J.lz - li.z;
-        } else {
-            ex = fmaf(oi.w, J.lx, -(J.m * li.x));
-            ey = fmaf(oi.w, J.ly, -(J.m * li.y));
-            ez = fmaf(oi.w, J.lz, -(J.m * li.z));
-        }
-        const float r = in ? fp2 * fmaf(dz, ez, fmaf(dy, ey, dx * ex)) : 0.0f;
-        const float wx = fmaf(f, ex, r * dx), wy = fmaf(f, ey, r * dy), wz = fmaf(f, ez, r * dz);
-        acc[0] += wx;
-        acc[1] += wy;
-        acc[2] += wz;
-        J.u0 -= wx;
-        J.u1 -= wy;
-        J.u2 -= wz;
-        return;
+    float ex, ey, ez;  // mu (equal masses: mu / m)
+    if constexpr (EQ) {
+        ex = J.lx - li.x;
+        ey = J.ly - li.y;
+        ez = J.lz - li.z;
+    } else {
+        ex = fmaf(oi.w, J.lx, -(J.m * li.x));
+        ey = fmaf(oi.w, J.ly, -(J.m * li.y));
+        ez = fmaf(oi.w, J.lz, -(J.m * li.z));
     }
-    const float dlj = fmaf(dz, J.lz, fmaf(dy, J.ly, dx * J.lx));
-    const float dli = fmaf(dz, li.z, fmaf(dy, li.y, dx * li.x));
-    float rr;
-    if constexpr (EQ)
-        rr = fp2 * (dlj - dli);
-    else
-        rr = fp2 * fmaf(oi.w, dlj, -(J.m * dli));
-    const float r = in ? rr : 0.0f;
-    const float mj = EQ ? 1.0f : J.m, mi = EQ ? 1.0f : oi.w;
-    // i side
-    acc[0] = fmaf(f, J.lx, acc[0]);
-    acc[1] = fmaf(f, J.ly, acc[1]);
-    acc[2] = fmaf(f, J.lz, acc[2]);
-    acc[3] = fmaf(mj, f, acc[3]);
-    acc[4] = fmaf(r, dx, acc[4]);
-    acc[5] = fmaf(r, dy, acc[5]);
-    acc[6] = fmaf(r, dz, acc[6]);
-    if constexpr (GM) acc[7] = fmaf(f, dlj, acc[7]);
-    // j side
-    J.u0 = fmaf(f, li.x, J.u0);
-    J.u1 = fmaf(f, li.y, J.u1);
-    J.u2 = fmaf(f, li.z, J.u2);
-    J.v = fmaf(mi, f, J.v);
-    J.x0 = fmaf(-r, dx, J.x0);
-    J.x1 = fmaf(-r, dy, J.x1);
-    J.x2 = fmaf(-r, dz, J.x2);
-    if constexpr (GM) J.g = fmaf(-f, dli, J.g);
+    const float r = in ? fp2 * fmaf(dz, ez, fmaf(dy, ey, dx * ex)) : 0.0f;
+    const float wx = fmaf(f, ex, r * dx), wy = fmaf(f, ey, r * dy), wz = fmaf(f, ez, r * dz);
+    acc[0] += wx;
+    acc[1] += wy;
+    acc[2] += wz;
+    J.w0 -= wx;
+    J.w1 -= wy;
+    J.w2 -= wz;
+    if constexpr (GM) {
+        acc[3] = fmaf(f, fmaf(dz, J.lz, fmaf(dy, J.ly, dx * J.lx)), acc[3]);
+        J.g = fmaf(-f, fmaf(dz, li.z, fmaf(dy, li.y, dx * li.x)), J.g);
+    }
 }
 
 // W rotation steps within groups of W lanes, as the force kernel's
@@ -146,17 +108,14 @@ __device__ __forceinline__ void rotate_block_adj(JAdj &J, const float4 (&oi)[IPL
     }
 }
 
-// j sums of a block to the float64 totals acc[c N + slot], c = U0 U1 U2 V X0 X1 X2 G
-// (the W form: W0 W1 W2).
+// j sums of a block to the float64 totals acc[c N + slot], c = W0 W1 W2 G.
 template <bool GM, bool EQ>
 __device__ __forceinline__ void flush_adj(const JAdj &J, double *acc, int64_t N)
 {
     constexpr int NC = adj_nacc(GM ? ADJOINT_GM : ADJOINT);
     if (J.slot < 0) return;
-    if (J.u0 == 0.f && J.u1 == 0.f && J.u2 == 0.f &&
-        (NC == 3 || (J.v == 0.f && J.x0 == 0.f && J.x1 == 0.f && J.x2 == 0.f)) && (!GM || J.g == 0.f))
-        return;
-    const float c[8] = {J.u0, J.u1, J.u2, J.v, J.x0, J.x1, J.x2, J.g};
+    if (J.w0 == 0.f && J.w1 == 0.f && J.w2 == 0.f && (!GM || J.g == 0.f)) return;
+    const float c[4] = {J.w0, J.w1, J.w2, J.g};
 #pragma unroll
     for (int k = 0; k < NC; ++k) atomicAdd(acc + k * N + J.slot, (double)c[k]);
 }
@@ -171,7 +130,7 @@ __device__ __forceinline__ void own_block_adj(const float4 (&oi)[IPL], const flo
 {
     constexpr unsigned SKIP = (0xFu << (B + 1)) & ((1u << IPL) - 1u);
     JAdj J{oi[B].x, oi[B].y, oi[B].z, oi[B].w, li[B].x, li[B].y, li[B].z,
-           0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, active[B] ? ib + 32 * B + lane : -1};
+           0.f, 0.f, 0.f, 0.f, active[B] ? ib + 32 * B + lane : -1};
     rotate_block_adj<IPL, GM, EQ, 1u << B, SKIP>(J, oi, li, K, p, lane);
     flush_adj<GM, EQ>(J, acc, N);
 }
@@ -209,7 +168,7 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
     if constexpr (HALF) {  // the chunk against itself on the low half-warp, 16 steps
         const bool lo = lane < 16;
         JAdj J{oi[0].x, oi[0].y, oi[0].z, oi[0].w, li[0].x, li[0].y, li[0].z,
-               0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, (lo && active[0]) ? ib + lane : -1};
+               0.f, 0.f, 0.f, 0.f, (lo && active[0]) ? ib + lane : -1};
         if (!lo) {
             J.x = J.y = J.z = FAR;
             J.m = J.lx = J.ly = J.lz = 0.f;
@@ -269,7 +228,7 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
             for (int b0 = 0; b0 < filled; b0 += 32) {
                 const int r = b0 + lane;
                 const int bend = min(filled, b0 + 32);
-                JAdj J{FAR, FAR, FAR, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -1};
+                JAdj J{FAR, FAR, FAR, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -1};
                 while (kk < ng && at < bend) {
                     const int cc = __shfl_sync(FULL, cnt, kk);
                     if (oo >= cc) {
@@ -346,14 +305,12 @@ __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, 
         if (!take_task(a, t, lane, task, a.order)) continue;
         const hacc_volume &vol = a.vols[task.w];
         bool ok = true;
-        // sub-chunks of larger tasks: 128 particles (four i per lane) in the W form,
-        // whose three sums leave the registers for it, else 64
-        constexpr int CHUNK = adj_wform(GM ? ADJOINT_GM : ADJOINT) ? 128 : 64;
+        // larger tasks: four i per lane, chunks of 128 particles
+        constexpr int CHUNK = 128;
         for (int sb = task.y; ok && sb < task.z; sb += CHUNK) {
             const int se = min(sb + CHUNK, task.z);
-            if (CHUNK == 128 && se - sb > 64)
-                ok = run_task_adj_sym<JT, STAGES, (CHUNK == 128 ? 4 : 2), GM, EQ>(a, ring, comp, acc, N, lane,
-                                                                                  task.x, sb, se, vol);
+            if (se - sb > 64)
+                ok = run_task_adj_sym<JT, STAGES, 4, GM, EQ>(a, ring, comp, acc, N, lane, task.x, sb, se, vol);
             else if (se - sb > 32)
                 ok = run_task_adj_sym<JT, STAGES, 2, GM, EQ>(a, ring, comp, acc, N, lane, task.x, sb, se, vol);
             else if (se - sb > 16)
@@ -370,43 +327,18 @@ __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, 
     }
 }
 
-// The W form: one component of dL/dx = W (equal masses: m W, m the common
-// mass) from the float64 totals, in input order; one component per launch
-// for the reason given at k_sym_finish.
-__global__ void __launch_bounds__(256)
-k_adj_sym_finish_w(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
-                   const float4 *__restrict__ pos, const uint32_t *mass_varies, float *__restrict__ out)
-{
-    const bool eq = mass_varies && *mass_varies == 0u;
-    const double sc = eq ? (double)pos[0].w : 1.0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-        out[__ldcs(perm + k)] = (float)(sc * __ldcs(acc + k));
-}
-
-// With dL/dm: dL/dx_k = m_k U - lam_k V + X (equal masses: m_k (U - lam_k V +
-// X)) and dL/dm_k = -G from the float64 totals, in input order.
+// One output component from its float64 totals, in input order: dL/dx = W
+// (equal masses: m W, m the common mass), dL/dm = -G (is_gm); one
+// component per launch for the reason given at k_sym_finish.
 __global__ void __launch_bounds__(256)
 k_adj_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
-                 const float4 *__restrict__ pos, const float4 *__restrict__ lam, const uint32_t *mass_varies,
-                 float *__restrict__ gx, float *__restrict__ gy, float *__restrict__ gz, float *__restrict__ gm)
+                 const float4 *__restrict__ pos, const uint32_t *mass_varies, bool is_gm,
+                 float *__restrict__ out)
 {
     const bool eq = mass_varies && *mass_varies == 0u;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int i = perm[k];
-        const double m = (double)pos[k].w;
-        const float4 l = lam[k];
-        const double V = acc[3 * N + k];
-        if (eq) {
-            gx[i] = (float)(m * (acc[k] - (double)l.x * V + acc[4 * N + k]));
-            gy[i] = (float)(m * (acc[N + k] - (double)l.y * V + acc[5 * N + k]));
-            gz[i] = (float)(m * (acc[2 * N + k] - (double)l.z * V + acc[6 * N + k]));
-        } else {
-            gx[i] = (float)(m * acc[k] - (double)l.x * V + acc[4 * N + k]);
-            gy[i] = (float)(m * acc[N + k] - (double)l.y * V + acc[5 * N + k]);
-            gz[i] = (float)(m * acc[2 * N + k] - (double)l.z * V + acc[6 * N + k]);
-        }
-        gm[i] = (float)(-acc[7 * N + k]);
-    }
+    const double sc = is_gm ? -1.0 : eq ? (double)pos[0].w : 1.0;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
+        out[__ldcs(perm + k)] = (float)(sc * __ldcs(acc + k));
 }
 
 template <int JT, int STAGES, bool GM, bool EQ>
@@ -472,7 +404,7 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
     a.lam = F.lam;
     a.counter = F.counter;
     HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
-    HACC_CUDA_TRY(cudaMemsetAsync(F.acc, 0, (size_t)mesh->N * (gm ? 8 : 3) * sizeof(double), st));
+    HACC_CUDA_TRY(cudaMemsetAsync(F.acc, 0, (size_t)mesh->N * (gm ? 4 : 3) * sizeof(double), st));
     hacc_launch L;
     if (launch) {
         L = *launch;
@@ -487,16 +419,10 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
     rc = gm ? launch_adj_sym<true>(a, F.acc, mesh->N, L, st) : launch_adj_sym<false>(a, F.acc, mesh->N, L, st);
     if (rc) return rc;
     const float4 *pos = reinterpret_cast<const float4 *>(binned->sorted4);
-    if (gm) {
-        k_adj_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc, binned->perm, pos, F.lam, binned->mass_varies, gx, gy,
-                                            gz, gm);
-        HACC_LAUNCH_CHECK();
-        return HACC_OK;
-    }
-    float *out[3] = {gx, gy, gz};
-    for (int c = 0; c < 3; ++c) {
-        k_adj_sym_finish_w<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, pos, binned->mass_varies,
-                                              out[c]);
+    float *out[4] = {gx, gy, gz, gm};
+    for (int c = 0; c < (gm ? 4 : 3); ++c) {
+        k_adj_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, pos, binned->mass_varies,
+                                            c == 3, out[c]);
         HACC_LAUNCH_CHECK();
     }
     return HACC_OK;
