@@ -20,7 +20,7 @@
 //   a += m_j f d
 // The accumulator is float32 within a tile and compensated (TwoSum into a
 // hi/lo pair) across tiles.
-#include "hacc_pairs.cuh"
+#include "hacc_hits.cuh"
 
 namespace hacc {
 namespace {
@@ -30,54 +30,11 @@ namespace {
 template <int MODE, int IPL>
 struct Acc;
 
-template <int IPL, int NC>
-struct AccN {
-    float a[IPL][NC], h[IPL][NC], l[IPL][NC];
-    __device__ __forceinline__ AccN()
-    {
-#pragma unroll
-        for (int u = 0; u < IPL; ++u)
-#pragma unroll
-            for (int k = 0; k < NC; ++k) a[u][k] = h[u][k] = l[u][k] = 0.f;
-    }
-    __device__ __forceinline__ void fold()
-    {
-#pragma unroll
-        for (int u = 0; u < IPL; ++u)
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                two_sum_acc(h[u][k], l[u][k], a[u][k]);
-                a[u][k] = 0.f;
-            }
-    }
-};
-
 template <int IPL>
 struct Acc<FORCE, IPL> : AccN<IPL, 3> {};
 
 template <int IPL>
 struct Acc<POTENTIAL, IPL> : AccN<IPL, 1> {};
-
-// One pair of the forward law, accumulated into acc[3] (EQ, equal masses:
-// f d, the mass applied to the total).  The cutoff test is a compare whose
-// predicate guards the three accumulating fma (no branch, no select): the
-// paper folds the same test into the loop with fsel (Sec. III).
-template <bool EQ>
-__device__ __forceinline__ void pair_force(const float4 p, float oxp, float oyp, float ozp, const PairConsts &K,
-                                           float *acc)
-{
-    float dx = p.x - oxp, dy = p.y - oyp, dz = p.z - ozp;
-    float se = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, K.eps)));
-    float t = rsqrt_hw(se);
-    float t2 = t * t;
-    float q = fmaf(fmaf(fmaf(fmaf(fmaf(K.nc[5], se, K.nc[4]), se, K.nc[3]), se, K.nc[2]), se, K.nc[1]), se,
-                   K.nc[0]);
-    float g = EQ ? fmaf(t2, t, q) : fmaf(t2, t, q) * p.w;
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %3, %4;\n\t"
-        "@p fma.rn.f32 %0, %5, %6, %0;\n\t@p fma.rn.f32 %1, %5, %7, %1;\n\t@p fma.rn.f32 %2, %5, %8, %2;\n\t}"
-        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2])
-        : "f"(se), "f"(K.rc2e), "f"(g), "f"(dx), "f"(dy), "f"(dz));
-}
 
 // Forward pair loop over one staged tile: every staged j meets the IPL i
 // particles of this lane.  Unrolled by hand, four j per trip.
@@ -103,27 +60,6 @@ __device__ __forceinline__ void tile_force(const float4 *__restrict__ tj, int n,
     }
 }
 
-// The short-range pair potential V(s) = pv(se) - (s + eps)^-1/2 (se = s + eps):
-// the integral of the force law, zero at the cutoff (F = -grad V).
-__device__ __forceinline__ float pair_potential_of(float se, const PairConsts &K)
-{
-    const float h = fmaf(fmaf(fmaf(fmaf(fmaf(fmaf(K.pv[6], se, K.pv[5]), se, K.pv[4]), se, K.pv[3]), se, K.pv[2]),
-                              se, K.pv[1]),
-                         se, K.pv[0]);
-    return h - rsqrt_hw(se);
-}
-
-__device__ __forceinline__ void pair_potential(const float4 p, float oxp, float oyp, float ozp, const PairConsts &K,
-                                               float *acc)
-{
-    float dx = p.x - oxp, dy = p.y - oyp, dz = p.z - ozp;
-    float se = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, K.eps)));
-    float v = pair_potential_of(se, K);
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, %2;\n\t@p fma.rn.f32 %0, %3, %4, %0;\n\t}"
-        : "+f"(acc[0])
-        : "f"(se), "f"(K.rc2e), "f"(p.w), "f"(v));
-}
-
 template <int IPL>
 __device__ __forceinline__ void tile_potential(const float4 *__restrict__ tj, int n, const float (&op)[IPL][3],
                                                const PairConsts &K, Acc<POTENTIAL, IPL> &A)
@@ -145,58 +81,6 @@ __device__ __forceinline__ void tile_potential(const float4 *__restrict__ tj, in
         for (int u = 0; u < IPL; ++u) pair_potential(p, op[u][0], op[u][1], op[u][2], K, A.a[u]);
     }
 }
-
-// One pair of the adjoint, accumulated into acc = (W, G) of one i: with f =
-// f_SR(s), fp2 = 2 f_SR'(s) and mu = m_i lam_j - m_j lam_i (equal masses, EQ:
-// mu / m = lam_j - lam_i),
-//   W += f mu + fp2 (d.mu) d      dL/dx_i = W (equal masses: m W)
-//   G += f (d.lam_j)              dL/dm_i = -G (GM only)
-// Summing the antisymmetric pair term takes the cancellation between the lam_j
-// and lam_i parts of a close pair out of the totals.
-template <bool GM, bool EQ>
-__device__ __forceinline__ void pair_adjoint(const float4 p, const float4 l, float oxp, float oyp, float ozp,
-                                             float mi, float lix, float liy, float liz, const PairConsts &K,
-                                             float (&acc)[ADJ_NACC])
-{
-    float dx = p.x - oxp, dy = p.y - oyp, dz = p.z - ozp;
-    float se = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, K.eps)));
-    float t = rsqrt_hw(se);
-    float t2 = t * t;
-    float t3 = t2 * t;
-    float q = fmaf(fmaf(fmaf(fmaf(fmaf(K.nc[5], se, K.nc[4]), se, K.nc[3]), se, K.nc[2]), se, K.nc[1]), se,
-                   K.nc[0]);
-    float f = t3 + q;
-    float qp = fmaf(fmaf(fmaf(fmaf(K.kp[4], se, K.kp[3]), se, K.kp[2]), se, K.kp[1]), se, K.kp[0]);
-    float fp2 = fmaf(-3.0f, t3 * t2, qp);
-    float ex, ey, ez;  // mu (equal masses: mu / m)
-    if constexpr (EQ) {
-        ex = l.x - lix;
-        ey = l.y - liy;
-        ez = l.z - liz;
-    } else {
-        ex = fmaf(mi, l.x, -(p.w * lix));
-        ey = fmaf(mi, l.y, -(p.w * liy));
-        ez = fmaf(mi, l.z, -(p.w * liz));
-    }
-    const float r = fp2 * fmaf(dz, ez, fmaf(dy, ey, dx * ex));
-    // the accumulations of this pair happen only inside the cutoff
-    if constexpr (GM) {
-        const float dlj = fmaf(dz, l.z, fmaf(dy, l.y, dx * l.x));
-        asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %4, %5;\n\t"
-            "@p fma.rn.f32 %0, %6, %7, %0;\n\t@p fma.rn.f32 %1, %6, %8, %1;\n\t@p fma.rn.f32 %2, %6, %9, %2;\n\t"
-            "@p fma.rn.f32 %0, %10, %11, %0;\n\t@p fma.rn.f32 %1, %10, %12, %1;\n\t"
-            "@p fma.rn.f32 %2, %10, %13, %2;\n\t@p fma.rn.f32 %3, %6, %14, %3;\n\t}"
-            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
-            : "f"(se), "f"(K.rc2e), "f"(f), "f"(ex), "f"(ey), "f"(ez), "f"(r), "f"(dx), "f"(dy), "f"(dz), "f"(dlj));
-    } else {
-        asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %3, %4;\n\t"
-            "@p fma.rn.f32 %0, %5, %6, %0;\n\t@p fma.rn.f32 %1, %5, %7, %1;\n\t@p fma.rn.f32 %2, %5, %8, %2;\n\t"
-            "@p fma.rn.f32 %0, %9, %10, %0;\n\t@p fma.rn.f32 %1, %9, %11, %1;\n\t@p fma.rn.f32 %2, %9, %12, %2;\n\t}"
-            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2])
-            : "f"(se), "f"(K.rc2e), "f"(f), "f"(ex), "f"(ey), "f"(ez), "f"(r), "f"(dx), "f"(dy), "f"(dz));
-    }
-}
-
 
 // Adjoint pair loop over one staged tile (positions tj, cotangents tl).
 template <int MODE, int IPL, bool EQ>
@@ -383,27 +267,14 @@ __device__ __forceinline__ bool run_task(const KArgs &a, Ring<MODE, JT, STAGES> 
 #pragma unroll
     for (int u = 0; u < IPL; ++u) {
         if (!active[u] || (half && lane >= 16)) continue;
-        const int o = a.perm[ib + il + 32 * u];
-        if constexpr (MODE == FORCE && EQ) {
-            a.out_x[o] = oi[u].w * (A.h[u][0] + A.l[u][0]);
-            a.out_y[o] = oi[u].w * (A.h[u][1] + A.l[u][1]);
-            a.out_z[o] = oi[u].w * (A.h[u][2] + A.l[u][2]);
-        } else if constexpr (MODE == FORCE) {
-            a.out_x[o] = A.h[u][0] + A.l[u][0];
-            a.out_y[o] = A.h[u][1] + A.l[u][1];
-            a.out_z[o] = A.h[u][2] + A.l[u][2];
-        } else if constexpr (MODE == POTENTIAL) {
-            // the sum met particle i itself once (d = 0, se = eps exactly): take that term out
-            const float self = pair_potential_of(K.eps, K);
-            a.out_x[o] = (A.h[u][0] + A.l[u][0]) - oi[u].w * self;
-        } else {
-            // dL/dx_i = W (equal masses: m W) ;  dL/dm_i = -G
-            const float sc = EQ ? oi[u].w : 1.0f;
-            a.out_x[o] = sc * A.total(u, 0);
-            a.out_y[o] = sc * A.total(u, 1);
-            a.out_z[o] = sc * A.total(u, 2);
-            if constexpr (MODE == ADJOINT_GM) a.out_m[o] = -A.total(u, 3);
-        }
+        auto total = [&](int k) {
+            if constexpr (is_adjoint(MODE)) {
+                if (EQ || k > 2) return A.total(u, k);
+                return A.total(u, k) - self_term(K, oi[u].w, k == 0 ? li[u].x : k == 1 ? li[u].y : li[u].z);
+            } else
+                return A.h[u][k] + A.l[u][k];
+        };
+        store_out<MODE>(a, a.perm[ib + il + 32 * u], oi[u], EQ, total);
     }
     return true;
 }
@@ -417,34 +288,10 @@ __device__ __forceinline__ bool run_task(const KArgs &a, Ring<MODE, JT, STAGES> 
 // memory, which caps it at 2 CTAs, so it may use up to 128 registers.
 __host__ __device__ constexpr int min_ctas(int mode) { return is_adjoint(mode) ? 2 : 3; }
 
-// EQ (force and adjoint): the equal-mass instantiation; as for the
-// symmetric kernel both are launched and the one that does not match the
-// flag returns.
+// The tasks of one launch, on the equal-mass (EQ) or the general path.
 template <int MODE, int JT, int STAGES, bool EQ>
-__global__ void __launch_bounds__(256, min_ctas(MODE)) k_pairs(const KArgs a)
+__device__ __forceinline__ void dense_tasks(const KArgs &a, Ring<MODE, JT, STAGES> &ring, float *comp, int lane)
 {
-    if constexpr (MODE != POTENTIAL) {
-        const bool eq = a.mass_varies && *a.mass_varies == 0u;
-        if (eq != EQ) return;
-    }
-    extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int WARP_BYTES = warp_smem_bytes(MODE, JT, STAGES);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char *wbase = smem + (size_t)warp * WARP_BYTES;
-    constexpr int TILE_BYTES = warp_tiles_bytes(MODE, JT, STAGES);
-    constexpr int COMP_BYTES = is_adjoint(MODE) ? ADJ_COMP_BYTES : 0;
-    Ring<MODE, JT, STAGES> ring;
-    ring.tiles = reinterpret_cast<float4 *>(wbase);
-    float *comp = reinterpret_cast<float *>(wbase + TILE_BYTES);
-    ring.bars = reinterpret_cast<uint64_t *>(wbase + TILE_BYTES + COMP_BYTES);
-
-    if (lane == 0) {
-        for (int s = 0; s < STAGES; ++s) mbar_init(smem_addr(&ring.bars[s]), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncwarp();
-
     const int ntask = task_count(a);
     while (true) {
         int t = 0;
@@ -452,7 +299,7 @@ __global__ void __launch_bounds__(256, min_ctas(MODE)) k_pairs(const KArgs a)
         t = __shfl_sync(FULL, t, 0);
         if (t >= ntask) break;
         int4 task;
-        if (!take_task(a, t, lane, task, a.order)) continue;
+        if (!take_task(a, a.order[t], lane, task)) continue;
         const hacc_volume &vol = a.vols[task.w];
         bool ok = true;
         // sub-chunks of larger tasks: 128 particles (four i per lane) for the adjoint, else 64
@@ -475,6 +322,66 @@ __global__ void __launch_bounds__(256, min_ctas(MODE)) k_pairs(const KArgs a)
     }
 }
 
+// The two mass paths share the kernel (the device flag picks one), and the
+// hit kernel behind it may start as soon as this one's blocks leave room.
+template <int MODE, int JT, int STAGES>
+__global__ void __launch_bounds__(256, min_ctas(MODE)) k_pairs(const KArgs a)
+{
+    allow_next_kernel();
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int WARP_BYTES = warp_smem_bytes(MODE, JT, STAGES);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned char *wbase = smem + (size_t)warp * WARP_BYTES;
+    constexpr int TILE_BYTES = warp_tiles_bytes(MODE, JT, STAGES);
+    constexpr int COMP_BYTES = is_adjoint(MODE) ? ADJ_COMP_BYTES : 0;
+    Ring<MODE, JT, STAGES> ring;
+    ring.tiles = reinterpret_cast<float4 *>(wbase);
+    float *comp = reinterpret_cast<float *>(wbase + TILE_BYTES);
+    ring.bars = reinterpret_cast<uint64_t *>(wbase + TILE_BYTES + COMP_BYTES);
+
+    if (lane == 0) {
+        for (int s = 0; s < STAGES; ++s) mbar_init(smem_addr(&ring.bars[s]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    if constexpr (MODE != POTENTIAL) {
+        if (a.mass_varies && *a.mass_varies == 0u) {
+            dense_tasks<MODE, JT, STAGES, true>(a, ring, comp, lane);
+            return;
+        }
+    }
+    dense_tasks<MODE, JT, STAGES, false>(a, ring, comp, lane);
+}
+
+// One hit-mask task (hacc_hits.cuh): at most 32 particles, outputs stored.
+template <int MODE>
+__device__ __forceinline__ bool hit_task(const KArgs &a, HitWarp &W, int lane, int c, int ib, int ie,
+                                         const hacc_volume &vol, bool eq)
+{
+    HitAcc<MODE> A;
+    float4 oi, li;
+    int i;
+    bool active;
+    if (!run_hits<MODE>(a, W.base, W.bar, W.phase, lane, c, ib, ie, vol, eq, false, A, oi, li, i, active)) return false;
+    if (active) store_out<MODE>(a, a.perm[i], oi, eq, [&](int k) { return A.total(k); });
+    return true;
+}
+
+// The tasks of the small cells (the back of the split list), by hit masks.
+template <int MODE>
+__global__ void __launch_bounds__(HITS_WARPS * 32, hits_ctas(MODE)) k_hits(const KArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    HitWarp W = hits_warp(smem, warp, lane, MODE);
+    const bool eq = MODE != POTENTIAL && a.mass_varies && *a.mass_varies == 0u;
+    hits_tasks(a, lane, [&](int c, int ib, int ie, const hacc_volume &vol) {
+        return hit_task<MODE>(a, W, lane, c, ib, ie, vol, eq);
+    });
+    wait_previous_kernel();
+}
+
 // Ordered pairs (j != i) inside the cutoff, decided exactly as the pair
 // kernels decide it (same offsets, same float32 s + eps, same compare).  One
 // warp per task, one i per lane, j read straight from global memory: a
@@ -488,7 +395,7 @@ k_count_pairs(const KArgs a, unsigned long long *__restrict__ total)
     unsigned long long cnt = 0;
     for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntask; t += warps) {
         int4 task;
-        if (!take_task(a, t, lane, task, nullptr)) continue;
+        if (!take_task(a, t, lane, task)) continue;
         const hacc_volume &vol = a.vols[task.w];
         const int n = vol.n;
         const float w = vol.w;
@@ -532,11 +439,11 @@ k_count_pairs(const KArgs a, unsigned long long *__restrict__ total)
 }
 
 
-template <int MODE, int JT, int STAGES, bool EQ>
-int launch_one(const KArgs &a, int warps, int ctas_per_sm, cudaStream_t st)
+template <int MODE, int JT, int STAGES>
+int launch_t(const KArgs &a, int warps, int ctas_per_sm, cudaStream_t st)
 {
     const size_t smem = (size_t)warps * warp_smem_bytes(MODE, JT, STAGES);
-    auto kern = k_pairs<MODE, JT, STAGES, EQ>;
+    auto kern = k_pairs<MODE, JT, STAGES>;
     if (smem > 48 * 1024)
         HACC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
@@ -548,20 +455,8 @@ int launch_one(const KArgs &a, int warps, int ctas_per_sm, cudaStream_t st)
     return HACC_OK;
 }
 
-template <int MODE, int JT, int STAGES>
-int launch_t(const KArgs &a, int warps, int ctas_per_sm, cudaStream_t st)
-{
-    if constexpr (MODE != POTENTIAL) {
-        if (a.mass_varies) {
-            const int rc = launch_one<MODE, JT, STAGES, true>(a, warps, ctas_per_sm, st);
-            if (rc) return rc;
-        }
-    }
-    return launch_one<MODE, JT, STAGES, false>(a, warps, ctas_per_sm, st);
-}
-
 template <int MODE>
-int launch_mode(const KArgs &a, const hacc_launch &L, cudaStream_t st)
+int launch_dense(const KArgs &a, const hacc_launch &L, cudaStream_t st)
 {
     const int wp = L.warps_per_cta, cps = L.ctas_per_sm;
 #define HACC_CASE(JT, S) \
@@ -570,6 +465,17 @@ int launch_mode(const KArgs &a, const hacc_launch &L, cudaStream_t st)
     HACC_CASE(128, 2) HACC_CASE(128, 3) HACC_CASE(128, 4) HACC_CASE(256, 2)
 #undef HACC_CASE
     return HACC_ERR_INVALID;
+}
+
+// Every task: the dense kernel's, then the small cells' by hit masks.
+template <int MODE>
+int launch_mode(KArgs a, const ForceWs &F, const hacc_launch &L, cudaStream_t st)
+{
+    int rc = split_tasks(a, F, true, st);
+    if (rc) return rc;
+    rc = launch_dense<MODE>(a, L, st);
+    if (rc || a.origin) return rc;
+    return launch_hits(k_hits<MODE>, MODE, st, a);
 }
 
 hacc_launch default_launch(int mode)
@@ -607,11 +513,9 @@ extern "C" int hacc_sr_force(const hacc_mesh *mesh, const hacc_binned *binned, c
     a.out_x = ax;
     a.out_y = ay;
     a.out_z = az;
-    a.counter = F.counter;
-    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
     hacc_launch L = launch ? *launch : default_launch(FORCE);
     a.wait_limit = wait_limit_of(L);
-    return launch_mode<FORCE>(a, L, st);
+    return launch_mode<FORCE>(a, F, L, st);
 }
 
 extern "C" int hacc_sr_force_adjoint(const hacc_mesh *mesh, const hacc_binned *binned, const hacc_lists *lists,
@@ -636,12 +540,10 @@ extern "C" int hacc_sr_force_adjoint(const hacc_mesh *mesh, const hacc_binned *b
     a.out_y = gy;
     a.out_z = gz;
     a.out_m = gm;
-    a.counter = F.counter;
-    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
     hacc_launch L = launch ? *launch : default_launch(ADJOINT);
     a.wait_limit = wait_limit_of(L);
-    if (gm) return launch_mode<ADJOINT_GM>(a, L, st);
-    return launch_mode<ADJOINT>(a, L, st);
+    if (gm) return launch_mode<ADJOINT_GM>(a, F, L, st);
+    return launch_mode<ADJOINT>(a, F, L, st);
 }
 
 extern "C" int hacc_sr_potential(const hacc_mesh *mesh, const hacc_binned *binned, const hacc_lists *lists,
@@ -656,11 +558,9 @@ extern "C" int hacc_sr_potential(const hacc_mesh *mesh, const hacc_binned *binne
     ForceWs F = force_layout(mesh, ws);
     KArgs a = base_args(mesh, binned, lists, p, status);
     a.out_x = phi;
-    a.counter = F.counter;
-    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
     hacc_launch L = launch ? *launch : default_launch(FORCE);
     a.wait_limit = wait_limit_of(L);
-    return launch_mode<POTENTIAL>(a, L, st);
+    return launch_mode<POTENTIAL>(a, F, L, st);
 }
 
 extern "C" int hacc_count_pairs(const hacc_mesh *mesh, const hacc_binned *binned, const hacc_lists *lists,

@@ -1,0 +1,618 @@
+// Pair sums by hit masks: the gather kernels' path for cells of few particles.
+//
+// In a near-uniform field only 15 % of a chaining-mesh cell's candidate pairs
+// lie inside the cutoff, so a loop over all candidates spends most of its
+// issue slots on pairs that add nothing.  Here a warp first finds the pairs
+// near or inside the cutoff with the tensor cores and then evaluates only
+// those:
+//   1. the j records of up to HITS_RECS candidates are staged in shared memory,
+//      shifted into the frame of the i cell, with n_j = (1 - delta) |x_j|^2;
+//   2. per 8 j and 16 i one mma.m16n8k8 (tf32) forms
+//      n_i + n_j - 2 x_i.x_j - (cut squared), whose sign bits are shifted into
+//      one 32-bit mask per (i, column of the 8);
+//   3. the masks are transposed so that every lane owns one i (with at most 16
+//      i, two lanes share one), and each lane walks its own set bits: one
+//      16-byte shared load and one pair term per bit, in the arithmetic and
+//      with the cutoff test of the dense loops.
+// The filter never loses a pair: tf32 rounds x to 2^-11 and n_j to 2^-11, so
+// the product sum is off by at most (2^-10 + 2^-11 + 2^-17)(|x_i|^2 + |x_j|^2)
+// (2 |x_i||x_j| <= |x_i|^2 + |x_j|^2; the last term covers the float32
+// accumulation), which delta = 2^-9 takes off in advance, and `cut` leaves
+// room for the rounding of s + eps in the exact test.  It admits about 1 %
+// more pairs than the test keeps.
+//
+// What bounds it: issue slots (70 % used) with the gathers' shared-memory
+// wavefronts close behind (58 %); per 32 pairs about 1.5 slots per candidate in
+// step 2 and 28 per hit in step 3, against 20 per candidate in the dense loop.
+// A batch whose fullest lane holds more hits than HITS_DENSE of its records (a
+// halo next door) is evaluated densely from the same tile instead.  Measured
+// (GB300), gather force and adjoint with dL/dm: 2.1M lattice particles 1.83 ->
+// 0.90 ms and 3.17 -> 1.42 ms, 4096 uniform ones 85 -> 68 us; 16.8M clustered
+// 63.2 -> 59.1 ms for the force, whose small cells alone take this path.
+#pragma once
+
+#include "hacc_terms.cuh"
+
+namespace hacc {
+namespace {
+
+constexpr int HITS_RECS = 256;  // staged candidates: 32 steps of 8 columns, one mask bit per step
+constexpr float HITS_DELTA = 0.001953125f;  // 2^-9
+// a batch is evaluated densely when its fullest lane has this share of hits
+constexpr float HITS_DENSE = 0.6f;
+
+// Chaining-mesh cells of at most HITS_CELL particles take the hit path (48 and
+// 96 measured within 5 % of 64 on lattice, uniform and clustered particles).
+constexpr int HITS_CELL = 64;
+
+// Shared memory of the path (bytes from its base): a pad of records outside
+// any cutoff (read by lanes that have run out of bits), the records, their
+// cotangents (adjoint), their n_j, and the mask words, each with the address
+// of its column.
+constexpr int HITS_PAD = 128;
+__host__ __device__ constexpr int hits_lam_off() { return HITS_PAD + HITS_RECS * 16; }
+__host__ __device__ constexpr int hits_n_off(int mode)
+{
+    return HITS_PAD + HITS_RECS * 16 * (is_adjoint(mode) ? 2 : 1);
+}
+__host__ __device__ constexpr int hits_word_off(int mode) { return hits_n_off(mode) + HITS_RECS * 4; }
+// ... eight words a lane and HITS_STOPS empty ones behind them
+constexpr int HITS_STOPS = 4;
+__host__ __device__ constexpr int hits_bytes(int mode) { return hits_word_off(mode) + (8 + HITS_STOPS) * 256; }
+
+__device__ __forceinline__ float4 lds128(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ float lds32(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts128(uint32_t a, float4 v)
+{
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void sts32(uint32_t a, float v)
+{
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y)
+{
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ uint32_t to_tf32(float x)
+{
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return r;
+}
+
+// d = A B: A 16 x 8 (lane (g, q) holds rows g, g + 8 of columns q, q + 4), B 8 x 8
+// (rows q, q + 4 of column g), d 16 x 8 (rows g, g + 8, columns 2 q, 2 q + 1).
+__device__ __forceinline__ void mma_16x8x8(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// a - b + s L rounded once (s = -1, 0, 1): two exact sums and their errors.
+__device__ __forceinline__ float image_delta(float a, float b, float sL)
+{
+    const float s1 = __fsub_rn(a, b), t1 = __fsub_rn(s1, a);
+    const float e1 = __fsub_rn(__fsub_rn(a, __fsub_rn(s1, t1)), __fadd_rn(b, t1));
+    const float s2 = __fadd_rn(s1, sL), t2 = __fsub_rn(s2, s1);
+    const float e2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, t2)), __fsub_rn(sL, t2));
+    return __fadd_rn(s2, __fadd_rn(e1, e2));
+}
+
+// Coordinates of a volume's cell (local id below 2^31, n^3 < 2^31).
+__device__ __forceinline__ void local_cell(uint32_t lc, uint32_t n, int &cx, int &cy, int &cz)
+{
+    const uint32_t r = lc / n, z = r / n;
+    cx = (int)(lc - r * n);
+    cy = (int)(r - z * n);
+    cz = (int)z;
+}
+
+// One i's sums: float32 over at most HITS_FOLD pairs, then compensated.
+constexpr int HITS_FOLD = 64;
+
+template <int MODE>
+struct HitAcc {
+    static constexpr int NC = MODE == FORCE ? 3 : MODE == POTENTIAL ? 1 : adj_nacc(MODE);
+    float p[ADJ_NACC], h[NC], l[NC];
+    __device__ __forceinline__ HitAcc()
+    {
+#pragma unroll
+        for (int k = 0; k < ADJ_NACC; ++k) p[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) h[k] = l[k] = 0.f;
+    }
+    __device__ __forceinline__ void fold()
+    {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            two_sum_acc(h[k], l[k], p[k]);
+            p[k] = 0.f;
+        }
+    }
+    __device__ __forceinline__ float total(int k) const { return h[k] + l[k]; }
+};
+
+// The pair (i, staged record at address rec), added to the i's sums.
+// One body serves both mass paths: with equal masses the staged masses and mi are 1.
+template <int MODE>
+__device__ __forceinline__ void hit_pair(uint32_t rec, const float4 &oi, float mi, const float4 &li, const PairConsts &K,
+                                         float (&p)[ADJ_NACC])
+{
+    const float4 o = lds128(rec);
+    if constexpr (MODE == FORCE)
+        pair_force<false>(o, oi.x, oi.y, oi.z, K, p);
+    else if constexpr (MODE == POTENTIAL)
+        pair_potential(o, oi.x, oi.y, oi.z, K, p);
+    else
+        pair_adjoint<MODE == ADJOINT_GM, false>(o, lds128(rec + HITS_RECS * 16), oi.x, oi.y, oi.z, mi, li.x, li.y,
+                                                li.z, K, p);
+}
+
+// The i particles [ib, ie) of chaining-mesh cell c (at most 32) against the
+// cell's list, all of it or the small cells (at most HITS_CELL particles)
+// only; unit: every mass taken as 1.  `phase`: the parity of the next use of `bar`.  On return lane (g, q)
+// = (lane / 4, lane mod 4) holds the totals of row g + 8 q (at most 16
+// particles: g + 8 (q mod 2), in both lanes that share the row), i = ib + row,
+// if active.  False if a wait ran out.
+template <int MODE>
+__device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t bar, uint32_t &phase, int lane,
+                                         int c, int ib, int ie, const hacc_volume &vol, bool unit, bool small_only,
+                                         HitAcc<MODE> &A,
+                                         float4 &oi, float4 &li, int &i_own, bool &active)
+{
+    const bool half = ie - ib <= 16;  // one tile of 16 rows, each row in two lanes; else two tiles
+    const int NW = half ? 4 : 8;      // mask words per lane
+    const PairConsts &K = a.k;
+    const uint32_t tile = base + HITS_PAD, words = base + hits_word_off(MODE) + 8 * lane,
+                   rows = words - 8 * lane;  // the i records, before the words are written
+    const int g = lane >> 2, q = lane & 3;
+    // the i records by one bulk copy (the previous task's use of the region is fenced at its end)
+    if (lane == 0) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(ie - ib) * 16u)
+                     : "memory");
+        bulk_copy(rows, a.pos + ib, (uint32_t)(ie - ib) * 16u, bar);
+    }
+    // records outside any cutoff ahead of the tile, and the end of the word list
+    if (lane < HITS_PAD / 16) sts128(base + 16 * lane, make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.f));
+    for (int k = 0; k < HITS_STOPS; ++k) sts64(words + (NW + k) * 256, 0u, tile);
+    const int row = g + 8 * (half ? q & 1 : q);
+    i_own = ib + row;
+    active = i_own < ie;
+    li = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (is_adjoint(MODE)) {
+        if (active) li = a.lam[i_own];
+    }
+
+    int cx, cy, cz;
+    local_cell((uint32_t)((int64_t)c - vol.cell_base), (uint32_t)vol.n, cx, cy, cz);
+    const float w = vol.w, ox = cell_centre(cx, w), oy = cell_centre(cy, w), oz = cell_centre(cz, w);
+
+    if (!warp_wait(bar, phase, a.wait_limit)) {
+        warp_wait(bar, phase, WAIT_LIMIT_CYCLES);  // let the copy in flight land
+        return false;
+    }
+    phase ^= 1u;
+    // A: rows (-2 x, -2 y, -2 z, 1 | n_i - cut in two tf32 words, 0, 0) against B's (x, y, z, n_j | 1, 1, 0, 0)
+    uint32_t Af[2][4];
+    oi = active ? lds128(rows + 16 * row) : make_float4(0.f, 0.f, 0.f, 0.f);
+    {
+        const float n2 = fmaf(oi.z, oi.z, fmaf(oi.y, oi.y, oi.x * oi.x));
+        const float ni = active ? fmaf(n2, 1.0f - HITS_DELTA, -K.hit_cut) : 1.0e30f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int rr = g + 8 * r;
+            const float x = q < 3 && ib + rr < ie ? lds32(rows + 16 * rr + 4 * q) : 0.f;
+            Af[r >> 1][r & 1] = to_tf32(q < 3 ? -2.0f * x : 1.0f);
+            const float n = __shfl_sync(FULL, ni, (lane & ~3) | r);  // half: rows below 16 only
+            const uint32_t hi = to_tf32(n);
+            Af[r >> 1][2 + (r & 1)] = q == 0 ? hi : q == 1 ? to_tf32(n - __uint_as_float(hi)) : 0u;
+        }
+    }
+    const float mi = unit ? 1.0f : oi.w;
+    const uint32_t ones = q < 2 ? __float_as_uint(1.0f) : 0u;
+
+    const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
+#pragma unroll 1
+    for (int64_t g0 = e0; g0 < e1; g0 += 32) {
+        // lane l describes one entry: its j range, image offset and place among the group's records.
+        // The 27-cell stencil is taken in steps of ten entries, so that every nine of them hold each
+        // x, each y and each z offset three times: a batch then holds about as many partners of every i.
+        const int ng = (int)min((int64_t)32, e1 - g0);
+        int jb = 0, cnt = 0;
+        float Dx = 0.f, Dy = 0.f, Dz = 0.f;
+        if (lane < ng) {
+            const int64_t e = g0 + (ng == 27 ? lane * 10 % 27 : lane);
+            const int cp = a.nbr_cell[e];
+            const int sh = a.nbr_shift[e];
+            jb = a.cell_start[cp];
+            cnt = a.cell_start[cp + 1] - jb;
+            if (small_only && cnt > HITS_CELL) cnt = 0;
+            int px, py, pz;
+            local_cell((uint32_t)((int64_t)cp - vol.cell_base), (uint32_t)vol.n, px, py, pz);
+            Dx = image_delta(cell_centre(px, w), ox, (float)(sh % 3 - 1) * vol.L);
+            Dy = image_delta(cell_centre(py, w), oy, (float)((sh / 3) % 3 - 1) * vol.L);
+            Dz = image_delta(cell_centre(pz, w), oz, (float)(sh / 9 - 1) * vol.L);
+        }
+        int first = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(FULL, first, o);
+            if (lane >= o) first += t;
+        }
+        const int total = __shfl_sync(FULL, first, 31);
+        first -= cnt;
+
+#pragma unroll 1
+        for (int t0 = 0; t0 < total; t0 += HITS_RECS) {
+            const int nb = min(HITS_RECS, total - t0), nb8 = (nb + 7) & ~7;
+            const int at = max(first, t0), n_own = min(first + cnt, t0 + HITS_RECS) - at;
+            const int base_j = jb - first + t0;  // record r of the batch is particle base_j + r of its entry
+            // ---- 1. stage the batch in the i cell's frame, U entries' loads in flight together
+            __syncwarp();  // the previous batch has been read
+            if (lane < nb8 - nb) {  // fill the last step with records outside any cutoff
+                sts128(tile + 16 * (nb + lane), make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.f));
+                sts32(base + hits_n_off(MODE) + 4 * (nb + lane), 1.0e30f);
+                if constexpr (is_adjoint(MODE))
+                    sts128(tile + HITS_RECS * 16 + 16 * (nb + lane), make_float4(0.f, 0.f, 0.f, 0.f));
+            }
+            auto put = [&](int r, const float4 &p, const float4 &l, int e) {
+                const float x = p.x + __shfl_sync(FULL, Dx, e), y = p.y + __shfl_sync(FULL, Dy, e),
+                            z = p.z + __shfl_sync(FULL, Dz, e);
+                if (r >= 0) {
+                    sts128(tile + 16 * r, make_float4(x, y, z, unit ? 1.0f : p.w));
+                    sts32(base + hits_n_off(MODE) + 4 * r, fmaf(z, z, fmaf(y, y, x * x)) * (1.0f - HITS_DELTA));
+                    if constexpr (is_adjoint(MODE)) sts128(tile + HITS_RECS * 16 + 16 * r, l);
+                }
+            };
+            constexpr int U = is_adjoint(MODE) ? 2 : 3;
+            const int place = (at - t0) | n_own << 16;
+            unsigned act = __ballot_sync(FULL, n_own > 0);
+#pragma unroll 1
+            while (act) {
+                float4 p[U], l[U];
+                int e[U], r[U], n[U], j[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    e[u] = __ffs(act) - 1;  // -1: none left
+                    act &= act - 1;
+                    const int pl = __shfl_sync(FULL, place, e[u]);
+                    n[u] = e[u] < 0 ? 0 : pl >> 16;
+                    r[u] = lane < n[u] ? (pl & 0xffff) + lane : -1;
+                    j[u] = __shfl_sync(FULL, base_j, e[u]) + (pl & 0xffff) + lane;
+                    p[u] = l[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (r[u] >= 0) {
+                        p[u] = a.pos[j[u]];
+                        if constexpr (is_adjoint(MODE)) l[u] = a.lam[j[u]];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) put(r[u], p[u], l[u], e[u]);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+#pragma unroll 1
+                    for (int o = 32; o < n[u]; o += 32) {
+                        const bool ok = lane + o < n[u];
+                        float4 p2 = make_float4(0.f, 0.f, 0.f, 0.f), l2 = p2;
+                        if (ok) {
+                            p2 = a.pos[j[u] + o];
+                            if constexpr (is_adjoint(MODE)) l2 = a.lam[j[u] + o];
+                        }
+                        put(ok ? r[u] + o : -1, p2, l2, e[u]);
+                    }
+                }
+            }
+            __syncwarp();
+            // ---- 2. sign masks: M[r][k] bit s = pair (row g + 8 r, record 8 s + 2 q + k) may be inside
+            uint32_t M[4][2];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) M[r][0] = M[r][1] = 0u;
+            {
+                const bool own_n = q == 3;
+                const uint32_t stride = own_n ? 32u : 128u;
+                uint32_t ad = (own_n ? base + hits_n_off(MODE) + 4 * g : tile + 16 * g + 4 * q) +
+                              stride * (uint32_t)(nb8 / 8 - 1);
+                auto signs = [&](int m, uint32_t b) {
+                    float d[4];
+                    mma_16x8x8(d, Af[m], b, ones);
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        M[2 * m][k] = __funnelshift_l(__float_as_uint(d[k]), M[2 * m][k], 1);
+                        M[2 * m + 1][k] = __funnelshift_l(__float_as_uint(d[2 + k]), M[2 * m + 1][k], 1);
+                    }
+                };
+                if (half) {
+#pragma unroll 2
+                    for (int s = nb8 / 8; s > 0; --s) {
+                        const uint32_t b = to_tf32(lds32(ad));
+                        ad -= stride;
+                        signs(0, b);
+                    }
+                } else {
+#pragma unroll 2
+                    for (int s = nb8 / 8; s > 0; --s) {
+                        const uint32_t b = to_tf32(lds32(ad));
+                        ad -= stride;
+                        signs(0, b);
+                        signs(1, b);
+                    }
+                }
+            }
+            // ---- transpose among the four lanes of a row group: the lane's own row, column by column.
+            // Lanes start at different columns, so that their gathers meet different banks.
+            int trips = 0;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (s >= 2 && half) break;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const uint32_t lo = (q ^ s) & 1 ? M[1][k] : M[0][k], hi = (q ^ s) & 1 ? M[3][k] : M[2][k];
+                    uint32_t v = !half && ((q ^ s) & 2) ? hi : lo;
+                    v = __shfl_xor_sync(FULL, v, s);
+                    trips += max(__popc(v), 1);
+                    sts64(words + 256 * ((2 * s + k) ^ (g & 1)), v, tile + 16 * (2 * (q ^ s) + k));
+                }
+            }
+            trips = __reduce_max_sync(FULL, trips);
+            __syncwarp();
+            // ---- 3. the pairs
+            if ((float)trips < HITS_DENSE * (float)(half ? nb8 / 2 : nb8)) {
+                uint32_t mask, col, wp = words + 256;
+                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mask), "=r"(col) : "r"(words) : "memory");
+                const uint32_t wend = words + NW * 256;
+                for (int f = 0; f < trips; f += HITS_FOLD) {
+                    if (f) A.fold();
+                    // trips in fours (a lane without bits reads the pad); a lane may run HITS_STOPS words
+                    // past its last before its pointer is put back
+#pragma unroll 1
+                    for (int t = min(trips - f, HITS_FOLD); t > 0; t -= HITS_STOPS) {
+#pragma unroll
+                        for (int u = 0; u < HITS_STOPS; ++u) {
+                            int b;
+                            uint32_t bit;
+                            asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(mask));   // -1: none (reads the pad)
+                            asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(b));  // clamped: 0 for none
+                            const uint32_t rec = col + 128 * b;
+                            mask &= ~bit;
+                            asm volatile(
+                                "{\n\t.reg .pred z;\n\tsetp.eq.u32 z, %0, 0;\n\t"
+                                "@z ld.shared.v2.u32 {%0, %1}, [%2];\n\t@z add.u32 %2, %2, 256;\n\t}"
+                                : "+r"(mask), "+r"(col), "+r"(wp)
+                                :
+                                : "memory");
+                            hit_pair<MODE>(rec, oi, mi, li, K, A.p);
+                        }
+                        wp = min(wp, wend);
+                    }
+                }
+            } else {
+                const int nr = half ? nb8 / 2 : nb8, r0 = half && (q & 2) ? nr : 0;
+                for (int f = 0; f < nr; f += HITS_FOLD) {
+                    if (f) A.fold();
+#pragma unroll 4
+                    for (int r = f; r < min(nr, f + HITS_FOLD); ++r)
+                        hit_pair<MODE>(tile + 16 * (r0 + r), oi, mi, li, K, A.p);
+                }
+            }
+            A.fold();
+        }
+    }
+    if (half) {
+        // lanes q and q ^ 2 hold the two parts of one row: the low one adds the high one's
+#pragma unroll
+        for (int k = 0; k < HitAcc<MODE>::NC; ++k) {
+            const float h2 = __shfl_xor_sync(FULL, A.h[k], 2), l2 = __shfl_xor_sync(FULL, A.l[k], 2);
+            two_sum_acc(A.h[k], A.l[k], h2);
+            A.l[k] = __fadd_rn(A.l[k], l2);
+        }
+        active = active && q < 2;
+    }
+    if constexpr (is_adjoint(MODE)) {
+        if (!unit) {
+            A.l[0] -= self_term(K, oi.w, li.x);
+            A.l[1] -= self_term(K, oi.w, li.y);
+            A.l[2] -= self_term(K, oi.w, li.z);
+        }
+    }
+    __syncwarp();
+    fence_async_proxy();  // the region's next use may be a bulk copy
+    return true;
+}
+
+// ---------------------------------------------------------------------------
+// Tasks: which cells take the path, and their persistent loop
+// ---------------------------------------------------------------------------
+
+// Which cells take the hit path: those of at most HITS_CELL particles and, in a
+// one-sided (gather) call, of at most 27 HITS_CELL candidates, since a larger
+// neighbour's pairs are mostly inside the cutoff or far outside and the dense
+// kernel holds two i per lane (without the second bound 1M clustered particles
+// take 5.4 ms, with it 4.2; the dense kernel alone 4.5).  (A symmetric call's dense tasks meet the large
+// neighbours themselves.)
+__device__ __forceinline__ bool hits_cell(const KArgs &a, int c, bool one_sided)
+{
+    if (a.cell_start[c + 1] - a.cell_start[c] > HITS_CELL) return false;
+    if (!one_sided) return true;
+    const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
+    int64_t nj = 0;
+    for (int64_t e = e0; e < e1; ++e) {
+#ifdef HACC_DEBUG_BOUNDS
+        if (a.nbr_cell[e] < 0 || a.nbr_cell[e] >= a.n_cells) continue;  // reported when the task is taken
+#endif
+        nj += a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
+    }
+    return nj <= 27 * HITS_CELL;
+}
+
+// Splits the heaviest-first task order in two, each about in that order:
+// the dense kernel's tasks from the front of `order`, the hit kernel's from
+// its back (N slots).  counts: [2] dense tasks, [3] hit tasks, zeroed before.
+__global__ void __launch_bounds__(1024)
+k_split_tasks(const KArgs a, bool one_sided, int32_t *__restrict__ order, int32_t *__restrict__ counts)
+{
+    __shared__ int wsum[2][32], base[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nt = task_count(a);
+    for (int t0 = blockIdx.x * 1024; t0 < nt; t0 += gridDim.x * 1024) {
+        const int t = t0 + threadIdx.x;
+        int oi = t < nt ? a.order[t] : -1, kind = -1;
+        if (t < nt) {
+#ifdef HACC_DEBUG_BOUNDS
+            const bool ok = oi >= 0 && oi < a.task_cap && a.tasks[oi].x >= 0 && a.tasks[oi].x < a.n_cells;
+            if (!ok) atomicOr(a.status, HACC_STATUS_BOUNDS);
+#else
+            constexpr bool ok = true;
+#endif
+            if (ok) kind = hits_cell(a, a.tasks[oi].x, one_sided) ? 1 : 0;
+        }
+        const unsigned m0 = __ballot_sync(FULL, kind == 0), m1 = __ballot_sync(FULL, kind == 1);
+        if (lane == 0) {
+            wsum[0][warp] = __popc(m0);
+            wsum[1][warp] = __popc(m1);
+        }
+        __syncthreads();
+        if (warp < 2) {
+            const int v = wsum[warp][lane];
+            int inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int n = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += n;
+            }
+            wsum[warp][lane] = inc - v;
+            if (lane == 31) base[warp] = inc ? atomicAdd(&counts[2 + warp], inc) : 0;
+        }
+        __syncthreads();
+        if (kind >= 0) {
+            const int64_t slot = base[kind] + wsum[kind][warp] + __popc((kind ? m1 : m0) & ((1u << lane) - 1u));
+            if (slot < a.N) order[kind ? a.N - 1 - slot : slot] = oi;
+        }
+        __syncthreads();  // wsum and base are reused
+    }
+}
+
+// Zeroes the task counters and, for chaining-mesh lists, splits the tasks:
+// `a` then names the dense kernel's order and count and the hit kernel's.
+int split_tasks(KArgs &a, const ForceWs &F, bool one_sided, cudaStream_t st)
+{
+    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, 4 * sizeof(int32_t), st));
+    a.counter = F.counter;
+    if (a.origin) return HACC_OK;  // tree lists: every task is the dense kernel's
+    int64_t g = (a.task_cap + 1023) / 1024;
+    if (g > num_sms() * 2) g = num_sms() * 2;
+    k_split_tasks<<<(int)(g < 1 ? 1 : g), 1024, 0, st>>>(a, one_sided, F.order, F.counter);
+    HACC_LAUNCH_CHECK();
+    a.order = F.order;
+    a.n_tasks = F.counter + 2;
+    a.hit_order = F.order + (a.N - 1);
+    a.hit_count = F.counter + 1;
+    return HACC_OK;
+}
+
+constexpr int HITS_WARPS = 4;
+__host__ __device__ constexpr int hits_ctas(int mode) { return is_adjoint(mode) ? 4 : 6; }
+__host__ __device__ constexpr int hits_warp_bytes(int mode)
+{
+    return (hits_bytes(mode) + 16 + 127) / 128 * 128;
+}
+
+struct HitWarp {
+    uint32_t base, bar, phase;
+};
+
+// A warp's region and its barrier, initialised.
+__device__ __forceinline__ HitWarp hits_warp(unsigned char *smem, int warp, int lane, int mode)
+{
+    HitWarp W;
+    W.base = smem_addr(smem + (size_t)warp * hits_warp_bytes(mode));
+    W.bar = W.base + hits_warp_bytes(mode) - 16;
+    W.phase = 0u;
+    if (lane == 0) {
+        mbar_init(W.bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_proxy();
+    }
+    __syncwarp();
+    return W;
+}
+
+// Persistent work-stealing loop: each warp takes hit tasks from a global
+// counter and runs them in chunks of at most 32 particles.
+template <class Run>
+__device__ __forceinline__ void hits_tasks(const KArgs &a, int lane, const Run &run)
+{
+    const int nt = a.hit_count[2];
+    while (true) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(a.hit_count, 1);
+        t = __shfl_sync(FULL, t, 0);
+        if (t >= nt) return;
+        int4 task;
+        if (!take_task(a, a.hit_order[-(int64_t)t], lane, task)) continue;
+        const hacc_volume &vol = a.vols[task.w];
+        for (int b = task.y; b < task.z; b += 32) {
+            if (!run(task.x, b, min(b + 32, task.z), vol)) {
+                if (lane == 0) atomicOr(a.status, HACC_STATUS_TIMEOUT);
+                return;
+            }
+        }
+    }
+}
+
+// Launched behind the dense kernel with programmatic serialisation: its
+// blocks fill the room that the dense kernel's leave, so that the two kernels'
+// last tasks overlap.  It needs nothing the dense kernel writes, and its
+// blocks wait for the dense kernel's end before they exit, so that work behind
+// it in the stream finds both done.
+template <class Kernel, class... Args>
+int launch_hits(Kernel kern, int mode, cudaStream_t st, Args... args)
+{
+    const int smem = HITS_WARPS * hits_warp_bytes(mode);
+    HACC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(num_sms() * hits_ctas(mode));
+    cfg.blockDim = dim3(HITS_WARPS * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    count_launch();
+    if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return HACC_ERR_CUDA;
+    }
+    return HACC_OK;
+}
+
+}  // namespace
+}  // namespace hacc

@@ -27,6 +27,7 @@ struct PairConsts {
     float rc2e;     // r_c^2 + eps (cut on se = s + eps)
     float nc[6];    // -(coefficients of poly~ in se), for f
     float kp[5];    // -2 (k+1) c~_{k+1}: Horner coefficients of -2 poly~'(se)
+    float hit_cut;  // no pair inside the cutoff has |x_j - x_i|^2 above this (with room for rounding)
     float pv[7];    // pair potential V = pv(se) - (se)^-1/2: degree-6 coefficients in se
 };
 
@@ -44,7 +45,9 @@ struct KArgs {
     const float4 *lam;   // sorted (lx, ly, lz, 0), adjoint only
     const int32_t *perm;
     float *out_x, *out_y, *out_z, *out_m;
-    int32_t *counter;
+    int32_t *counter;    // tasks taken
+    int32_t *hit_count;  // mesh lists: the tasks taken by, and the number of, the hit kernel
+    const int32_t *hit_order;  // its tasks, from this slot downwards
     uint32_t *status;
     PairConsts k;
     const uint32_t *mass_varies;  // 0: every mass equal (the equal-mass force paths); NULL: general
@@ -94,6 +97,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// Programmatic launch order: lets a kernel launched behind this one (with the
+// serialisation attribute) start in the room this one leaves, and waits there
+// until this one has finished and its writes are visible.
+__device__ __forceinline__ void allow_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // All lanes wait for a barrier phase; false (uniformly) once the wait has
 // lasted `limit` clock64 cycles of lane 0, checked before every poll.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long long limit)
@@ -107,8 +116,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long lo
     }
 }
 
-// The number of tasks to run, and task t of the heaviest-first order, with
-// whether it may be run.  A product build just reads them.  A debug build
+// The number of tasks to run, and task oi of the task buffer, with whether it
+// may be run.  A product build just reads them.  A debug build
 // (HACC_DEBUG_BOUNDS) first checks every index the task leads to -- the task
 // count against the task buffer, its order entry and record, its volume, and
 // on a chaining mesh its cell, its slot range and each entry of the cell's
@@ -128,13 +137,12 @@ __device__ __forceinline__ int task_count(const KArgs &a)
     return nt;
 }
 
-__device__ __forceinline__ bool take_task(const KArgs &a, int t, int lane, int4 &task, const int32_t *order)
+__device__ __forceinline__ bool take_task(const KArgs &a, int oi, int lane, int4 &task)
 {
 #ifndef HACC_DEBUG_BOUNDS
-    task = a.tasks[order ? order[t] : t];
+    task = a.tasks[oi];
     return true;
 #else
-    const int oi = order ? order[t] : t;
     bool ok = oi >= 0 && oi < a.task_cap;
     task = ok ? a.tasks[oi] : make_int4(0, 0, 0, 0);
     ok = ok && task.w >= 0 && task.w < a.V;
@@ -345,6 +353,8 @@ void pair_consts(const hacc_sr_params *p, PairConsts &K)
     }
     K.eps = p->eps;
     K.rc2e = (float)((double)p->rcut * (double)p->rcut + (double)p->eps);
+    // s + eps < r_c^2 + eps in float32 admits s up to r_c^2 plus the rounding of s and of the sum
+    K.hit_cut = (float)((double)p->rcut * (double)p->rcut * (1.0 + 1.0 / 4096) + (double)p->eps / (1 << 20));
     for (int k = 0; k < 6; ++k) K.nc[k] = (float)(-ct[k]);
     for (int k = 0; k < 5; ++k) K.kp[k] = (float)(-2.0 * (k + 1) * ct[k + 1]);
     // potential: V(s) = C0 - (s + eps)^-1/2 - P(s) / 2 with P(s) = sum_k c_k s^(k+1) / (k+1),
@@ -367,12 +377,14 @@ void pair_consts(const hacc_sr_params *p, PairConsts &K)
 }
 
 // Workspace of the pair calls: the task counter, the adjoints' sorted
-// cotangents (16 B per particle), and the symmetric kernels' float64 sums
-// (3 per particle for the force, 3 or 4 for the adjoint).
+// cotangents (16 B per particle), the symmetric kernels' float64 sums
+// (3 per particle for the force, 3 or 4 for the adjoint), and the split task order
+// (4 B per particle: a task holds at least one).
 constexpr int SYM_ACC_MAX = 4;
 
 struct ForceWs {
-    int32_t *counter;
+    int32_t *counter;  // the dense and the hit kernel's task counters and task counts
+    int32_t *order;    // the split task order (hacc_hits.cuh), one slot per particle
     float4 *lam;
     double *acc;
     size_t total;
@@ -386,7 +398,9 @@ ForceWs force_layout(const hacc_mesh *mesh, void *ws)
     F.counter = reinterpret_cast<int32_t *>(p);
     F.lam = reinterpret_cast<float4 *>(p ? p + 256 : nullptr);
     F.acc = reinterpret_cast<double *>(p ? p + 256 + lam_bytes : nullptr);
-    F.total = 256 + lam_bytes + round_up((size_t)mesh->N * 8 * SYM_ACC_MAX, 256);
+    const size_t acc_bytes = round_up((size_t)mesh->N * 8 * SYM_ACC_MAX, 256);
+    F.order = reinterpret_cast<int32_t *>(p ? p + 256 + lam_bytes + acc_bytes : nullptr);
+    F.total = 256 + lam_bytes + acc_bytes + round_up((size_t)mesh->N * 4, 256);
     return F;
 }
 

@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sym(const KArgs a, double *acc
         t = __shfl_sync(FULL, t, 0);
         if (t >= ntask) break;
         int4 task;
-        if (!take_task(a, t, lane, task, a.order)) continue;
+        if (!take_task(a, a.order[t], lane, task)) continue;
         const hacc_volume &vol = a.vols[task.w];
         bool ok;
         const int size = task.z - task.y;

@@ -1,0 +1,102 @@
+"""The hit path of the pair kernels (chaining-mesh cells of few particles).
+
+Cells of n particles each at the edges of its row tiles (8, 16, 32), of the
+cell size it takes (64 and 65) and of its batches of 256 candidates (27 cells
+of 9 and 10, a last step of one record), small cells around one large cell
+(both kernels add to the same particles), and a fine mesh whose lists span
+several groups of 32 entries.  Every pair call on both mass paths against the
+float64 oracle; the gather calls again bit for bit."""
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import MAX_TOL, RMS_TOL, err_norms, need_cuda
+from synth import default_coeffs
+
+pytestmark = pytest.mark.gpu
+
+EPS, RC = 0.01, 3.0
+
+
+def cells(n, side, big=0, seed=0, L=None):
+    """n particles in every cell of width 3 (side^3 of them), big more in one."""
+    rng = np.random.default_rng(seed)
+    g = np.stack(np.meshgrid(*[np.arange(side)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    own = np.repeat(g, n, axis=0)
+    own = np.concatenate([own, np.tile(g[len(g) // 2], (big, 1))])
+    pos = (own + rng.uniform(0.001, 0.999, own.shape)) * 3.0
+    return pos[rng.permutation(len(pos))].astype(np.float32), 3.0 * side
+
+
+def rounding_bounds(pos, m, lam, L):
+    """Per particle, what the rounding of its pairs' terms can add to a force and to a gradient component.  With t =
+    (s + eps)^-1/2 from a root within two units in the last place, t^3 is off by 2^-21 of itself and a Horner sum of
+    terms whose magnitudes add to at most 6 (value) or 8 (slope times s) by 6 2^-24 of them; the offsets, below 8 in
+    magnitude, add 2^-22 to a distance."""
+    d = pos[None] - pos[:, None]
+    d -= L * np.round(d / L)
+    s = (d * d).sum(-1)
+    t = (s + EPS) ** -0.5
+    near = (s < RC * RC) & (s > 0)
+    f = 2.0 ** -21 * (t ** 3 + 6) * np.sqrt(s) + 2.0 ** -22 * 4 * (t ** 3 + 1)
+    slope = 2.0 ** -21 * (8 * t ** 3 + 16) + 2.0 ** -22 * 16 * (t ** 4 + 1)
+    l = np.linalg.norm(lam, axis=1)
+    mu = m[:, None] * l[None] + m[None] * l[:, None]
+    return (near * m[None] * f).sum(1), (near * mu * slope).sum(1)
+
+
+CASES = [(1, 3, 0, 3.0, 32), (8, 3, 0, 3.0, 32), (9, 3, 0, 3.0, 32), (10, 4, 0, 3.0, 64), (16, 3, 0, 3.0, 32),
+         (17, 3, 0, 3.0, 32), (32, 3, 0, 3.0, 32), (33, 3, 0, 3.0, 32), (33, 3, 0, 3.0, 64), (64, 3, 0, 3.0, 128),
+         (65, 3, 0, 3.0, 128), (12, 3, 300, 3.0, 128), (20, 3, 70, 3.0, 32), (19, 4, 0, 1.5, 32), (3, 3, 0, 0.75, 32)]
+
+
+@pytest.mark.parametrize("n,side,big,cell_min,split_T", CASES)
+@pytest.mark.parametrize("masses", ["equal", "varied"])
+def test_cells_of_every_size(n, side, big, cell_min, split_T, masses):
+    torch = need_cuda()
+    import paper_1211_4864_gb300 as hs
+    hs.load()
+    pos, L = cells(n, side, big, seed=n + big)
+    N = len(pos)
+    rng = np.random.default_rng(5)
+    m = rng.uniform(0.5, 2.0, N).astype(np.float32) if masses == "varied" else np.full(N, 0.37, np.float32)
+    lam = rng.normal(size=(N, 3)).astype(np.float32)
+    c = default_coeffs(RC, EPS)
+    prm = hs.SRParams(EPS, RC, c)
+    sr = hs.ShortRange(L, np.array([0, N]), RC, cell_min=cell_min, split_T=split_T)
+    p = torch.tensor(pos.T.copy(), device="cuda")
+    lt = torch.tensor(lam.T.copy(), device="cuda")
+    sr.prepare(p, torch.tensor(m, device="cuda"))
+    a, phi = sr.force(prm), sr.potential(prm)
+    g, gm = sr.adjoint(prm, lt)
+    got = {"force": a, "symmetric": sr.force_symmetric(prm), "adjoint": g, "adjoint w": sr.adjoint(prm, lt, want_gm=False)[0]}
+    gs, gms = sr.adjoint_symmetric(prm, lt)
+    got["adjoint symmetric"] = gs
+    got["adjoint symmetric w"] = sr.adjoint_symmetric(prm, lt, want_gm=False)[0]
+    again = sr.force(prm)
+    torch.cuda.synchronize()
+    sr.check_status()
+    c64 = c.astype(np.float64)
+    A = oracle.sr_force(*pos.T.copy(), m, L, EPS, RC, c64)
+    G, GM = oracle.sr_force_adjoint(*pos.T.copy(), m, L, EPS, RC, c64, lam.astype(np.float64))
+    P = oracle.sr_potential(*pos.T.copy(), m, L, EPS, RC, c64)
+    if n < 8:  # few pairs, most of them where f = t^3 - poly nearly cancels: the terms' own rounding
+        bf, bg = rounding_bounds(pos.astype(np.float64), m, lam, L)
+        for name, t in got.items():
+            err = np.abs(t.cpu().numpy().T - (G if "adjoint" in name else A)).max(1)
+            assert np.all(err <= (bg if "adjoint" in name else bf) + 1e-9), name
+    else:
+        for name, t in got.items():
+            rms, mx = err_norms(t.cpu().numpy().T.astype(np.float64), G if "adjoint" in name else A)
+            assert rms < RMS_TOL and mx < MAX_TOL, (name, rms, mx)
+        for name, t in (("adjoint gm", gm), ("adjoint symmetric gm", gms)):
+            rms = np.linalg.norm(t.cpu().numpy() - GM) / np.linalg.norm(GM)
+            assert rms < RMS_TOL, (name, rms)
+    # V = poly(se) - se^-1/2: eight Horner steps of terms below 1.5 and a root within two units in the last
+    # place, so a pair is off by at most 8 2^-24 1.5 + 2^-22 (|V| + 1.5)
+    bound = (8 * 1.5 * 2.0 ** -24 + 1.5 * 2.0 ** -22) * m.sum() + 2.0 ** -22 * np.abs(P)
+    assert np.all(np.abs(phi.cpu().numpy() - P) < bound), "potential"
+    if n >= 8:
+        assert np.linalg.norm(phi.cpu().numpy() - P) / np.linalg.norm(P) < RMS_TOL
+    assert torch.equal(a, again)
