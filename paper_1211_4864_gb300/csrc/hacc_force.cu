@@ -292,14 +292,14 @@ __host__ __device__ constexpr int min_ctas(int mode) { return is_adjoint(mode) ?
 template <int MODE, int JT, int STAGES, bool EQ>
 __device__ __forceinline__ void dense_tasks(const KArgs &a, Ring<MODE, JT, STAGES> &ring, float *comp, int lane)
 {
-    const int ntask = task_count(a);
+    const int ntask = *a.n_items;
     while (true) {
         int t = 0;
         if (lane == 0) t = atomicAdd(a.counter, 1);
         t = __shfl_sync(FULL, t, 0);
         if (t >= ntask) break;
         int4 task;
-        if (!take_task(a, a.order[t], lane, task)) continue;
+        if (!take_task(a, a.items[t].x, lane, task)) continue;
         const hacc_volume &vol = a.vols[task.w];
         bool ok = true;
         // sub-chunks of larger tasks: 128 particles (four i per lane) for the adjoint, else 64

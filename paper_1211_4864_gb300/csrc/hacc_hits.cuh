@@ -29,6 +29,7 @@
 // (GB300), gather force and adjoint with dL/dm: 2.1M lattice particles 1.83 ->
 // 0.90 ms and 3.17 -> 1.42 ms, 4096 uniform ones 85 -> 68 us; 16.8M clustered
 // 63.2 -> 59.1 ms for the force, whose small cells alone take this path.
+// Symmetric force and adjoint, lattice: 1.24 -> 0.91 ms and 2.20 -> 1.35 ms.
 #pragma once
 
 #include "hacc_terms.cuh"
@@ -41,9 +42,11 @@ constexpr float HITS_DELTA = 0.001953125f;  // 2^-9
 // a batch is evaluated densely when its fullest lane has this share of hits
 constexpr float HITS_DENSE = 0.6f;
 
-// Chaining-mesh cells of at most HITS_CELL particles take the hit path (48 and
-// 96 measured within 5 % of 64 on lattice, uniform and clustered particles).
-constexpr int HITS_CELL = 64;
+// Chaining-mesh cells of at most HITS_CELL particles take the hit path.  40,
+// 48, 64 and 96 measured within 6 % of each other on lattice, uniform and
+// clustered particles (symmetric lattice force 0.94, 0.91 ms at 40, 64; 1.24
+// with the dense kernel alone); 40 covers the cells of a near-uniform field.
+constexpr int HITS_CELL = 40;
 
 // Shared memory of the path (bytes from its base): a pad of records outside
 // any cutoff (read by lanes that have run out of bits), the records, their
@@ -471,31 +474,119 @@ __device__ __forceinline__ bool hits_cell(const KArgs &a, int c, bool one_sided)
     return nj <= 27 * HITS_CELL;
 }
 
-// Splits the heaviest-first task order in two, each about in that order:
-// the dense kernel's tasks from the front of `order`, the hit kernel's from
-// its back (N slots).  counts: [2] dense tasks, [3] hit tasks, zeroed before.
+// Segments.  In a symmetric call the sums of a task go to the totals by
+// atomics, so a task may be cut along its j records: without that one warp
+// holds a halo cell's task of 128 particles and ten thousand j for over a
+// millisecond, and the kernel's last tasks leave the GPU idle.  A task of
+// more than a.seg_pairs pairs becomes segments of about that many (at most
+// one per particle of the task, and 256 j at least).  An item of the dense
+// kernels is (task, segment | scale << 16 | last << 24): segment s of scale k
+// holds the j records [s per, (s + 1) per), per = segment_records 2^k, the
+// last one all the rest.
+constexpr int SEG_WHOLE = 1 << 24;  // segment 0 and the last: the whole task
+__device__ __forceinline__ int segment_records(const KArgs &a, int size) { return max(a.seg_pairs / size, 256) & ~31; }
+__device__ __forceinline__ int segment_count(const KArgs &a, int size, int nj, int &scale)
+{
+    const int most = min(size, 32767), per = segment_records(a, size);
+    scale = 0;
+    while ((nj + (per << scale) - 1) / (per << scale) > most) ++scale;
+    return max(1, (nj + (per << scale) - 1) / (per << scale));
+}
+
+// Pairs per segment for N particles: the tail costs a share of the whole
+// call, the segments' own prologues and sums a share of the pairs.  Symmetric
+// force with segments of 16k, 32k, 64k, 128k pairs: 262,144 clustered particles
+// 0.40, 0.40, 0.42, 0.53 ms (0.56 uncut), 16.8M 38.9, 38.8, 37.6, 37.1 ms; with
+// this rule 0.40 and 34.9 ms (36.3 uncut), 1M 3.8 -> 2.8 ms.
+int seg_pairs_for(int64_t N)
+{
+    const int64_t p = N / 16;
+    return (int)(p < 32768 ? 32768 : p > (1 << 20) ? (1 << 20) : p);
+}
+
+// The list entry of cell (or leaf) c itself, image 13.  A chaining-mesh list
+// is symmetric under d -> -d with the cell in the middle; a tree leaf's list
+// is sorted by (image code, leaf id) and symmetric too (leaf j with image s
+// is listed for i iff i with image -s is listed for j), so its own entry is
+// found by bisection and everything after it is the forward half.
+__device__ __forceinline__ int64_t self_entry(const KArgs &a, int c, int64_t e0, int64_t e1, const hacc_volume &vol)
+{
+    if (!a.origin) return e0 + (vol.S - 1) / 2;
+    int64_t lo = e0, hi = e1 - 1;
+    while (lo < hi) {  // first entry with (code, leaf) >= (13, c)
+        const int64_t mid = (lo + hi) >> 1;
+        const int code = a.nbr_shift[mid], leaf = a.nbr_cell[mid];
+        if (code < 13 || (code == 13 && leaf < c)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Which half of its list a symmetric call's dense task walks: every entry
+// after its own cell, and the small cells before it -- those cells' tasks run
+// on the hit path, which sums small cells only, so a dense cell meets all of
+// its small neighbours itself (both particles of each pair).
+__device__ __forceinline__ int64_t first_entry(const KArgs &a, int64_t e0, int64_t mid) { return a.origin ? mid : e0; }
+__device__ __forceinline__ bool takes_entry(int64_t e, int64_t mid, int cnt) { return e > mid || cnt <= HITS_CELL; }
+
+// The j records a symmetric call's dense task meets beyond its own chunk.
+__device__ __forceinline__ int dense_reach(const KArgs &a, const int4 &task)
+{
+    const int64_t e0 = a.nbr_off[task.x], e1 = a.nbr_off[task.x + 1];
+    const int64_t mid = self_entry(a, task.x, e0, e1, a.vols[task.w]);
+    int64_t nj = a.cell_start[task.x + 1] - task.z;
+    for (int64_t e = first_entry(a, e0, mid); e < e1; ++e) {
+        if (e == mid) continue;
+#ifdef HACC_DEBUG_BOUNDS
+        if (!a.origin && (a.nbr_cell[e] < 0 || a.nbr_cell[e] >= a.n_cells)) continue;  // reported when taken
+#endif
+        const int cnt = a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
+        if (takes_entry(e, mid, cnt)) nj += cnt;
+    }
+    return (int)min(max(nj, (int64_t)0), (int64_t)1 << 30);
+}
+
+// Splits the heaviest-first task order in two, each about in that order: the
+// dense kernel's items from the front of `items`, the hit kernel's tasks from
+// its back (N slots).  counts: [2] items, [3] hit tasks, zeroed before.
 __global__ void __launch_bounds__(1024)
-k_split_tasks(const KArgs a, bool one_sided, int32_t *__restrict__ order, int32_t *__restrict__ counts)
+k_split_tasks(const KArgs a, bool one_sided, int2 *__restrict__ items, int32_t *__restrict__ counts)
 {
     __shared__ int wsum[2][32], base[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nt = task_count(a);
     for (int t0 = blockIdx.x * 1024; t0 < nt; t0 += gridDim.x * 1024) {
         const int t = t0 + threadIdx.x;
-        int oi = t < nt ? a.order[t] : -1, kind = -1;
+        const int oi = t < nt ? a.order[t] : -1;
+        int kind = 0, n = 0, scale = 0;  // items of the thread's task, for the dense (0) or the hit kernel (1)
         if (t < nt) {
+            bool ok = true;
 #ifdef HACC_DEBUG_BOUNDS
-            const bool ok = oi >= 0 && oi < a.task_cap && a.tasks[oi].x >= 0 && a.tasks[oi].x < a.n_cells;
+            ok = oi >= 0 && oi < a.task_cap;
+            if (ok) {
+                const int4 task = a.tasks[oi];
+                ok = task.w >= 0 && task.w < a.V && task.y < task.z && task.x >= 0 &&
+                     (a.origin || task.x < a.n_cells);
+            }
             if (!ok) atomicOr(a.status, HACC_STATUS_BOUNDS);
-#else
-            constexpr bool ok = true;
 #endif
-            if (ok) kind = hits_cell(a, a.tasks[oi].x, one_sided) ? 1 : 0;
+            if (ok) {
+                const int4 task = a.tasks[oi];
+                kind = !a.origin && hits_cell(a, task.x, one_sided) ? 1 : 0;
+                n = kind || one_sided ? 1 : segment_count(a, task.z - task.y, dense_reach(a, task), scale);
+            }
         }
-        const unsigned m0 = __ballot_sync(FULL, kind == 0), m1 = __ballot_sync(FULL, kind == 1);
-        if (lane == 0) {
-            wsum[0][warp] = __popc(m0);
-            wsum[1][warp] = __popc(m1);
+        int before[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int v = kind == k ? n : 0;
+            int inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int s = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += s;
+            }
+            before[k] = inc - v;
+            if (lane == 31) wsum[k][warp] = inc;
         }
         __syncthreads();
         if (warp < 2) {
@@ -503,35 +594,34 @@ k_split_tasks(const KArgs a, bool one_sided, int32_t *__restrict__ order, int32_
             int inc = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int n = __shfl_up_sync(FULL, inc, o);
-                if (lane >= o) inc += n;
+                const int s = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += s;
             }
             wsum[warp][lane] = inc - v;
             if (lane == 31) base[warp] = inc ? atomicAdd(&counts[2 + warp], inc) : 0;
         }
         __syncthreads();
-        if (kind >= 0) {
-            const int64_t slot = base[kind] + wsum[kind][warp] + __popc((kind ? m1 : m0) & ((1u << lane) - 1u));
-            if (slot < a.N) order[kind ? a.N - 1 - slot : slot] = oi;
-        }
+        const int64_t slot = (int64_t)base[kind] + wsum[kind][warp] + before[kind];
+        for (int s = 0; s < n; ++s)
+            if (slot + s < a.N) items[kind ? a.N - 1 - slot : slot + s] = make_int2(oi, s | scale << 16 | (s == n - 1 ? 1 << 24 : 0));
         __syncthreads();  // wsum and base are reused
     }
 }
 
-// Zeroes the task counters and, for chaining-mesh lists, splits the tasks:
-// `a` then names the dense kernel's order and count and the hit kernel's.
+// Zeroes the task counters and splits the tasks: `a` then names the dense
+// kernel's items and the hit kernel's tasks.
 int split_tasks(KArgs &a, const ForceWs &F, bool one_sided, cudaStream_t st)
 {
     HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, 4 * sizeof(int32_t), st));
     a.counter = F.counter;
-    if (a.origin) return HACC_OK;  // tree lists: every task is the dense kernel's
+    a.seg_pairs = seg_pairs_for(a.N);
     int64_t g = (a.task_cap + 1023) / 1024;
     if (g > num_sms() * 2) g = num_sms() * 2;
-    k_split_tasks<<<(int)(g < 1 ? 1 : g), 1024, 0, st>>>(a, one_sided, F.order, F.counter);
+    k_split_tasks<<<(int)(g < 1 ? 1 : g), 1024, 0, st>>>(a, one_sided, F.items, F.counter);
     HACC_LAUNCH_CHECK();
-    a.order = F.order;
-    a.n_tasks = F.counter + 2;
-    a.hit_order = F.order + (a.N - 1);
+    a.items = F.items;
+    a.n_items = F.counter + 2;
+    a.hit_order = F.items + (a.N - 1);
     a.hit_count = F.counter + 1;
     return HACC_OK;
 }
@@ -575,7 +665,7 @@ __device__ __forceinline__ void hits_tasks(const KArgs &a, int lane, const Run &
         t = __shfl_sync(FULL, t, 0);
         if (t >= nt) return;
         int4 task;
-        if (!take_task(a, a.hit_order[-(int64_t)t], lane, task)) continue;
+        if (!take_task(a, a.hit_order[-(int64_t)t].x, lane, task)) continue;
         const hacc_volume &vol = a.vols[task.w];
         for (int b = task.y; b < task.z; b += 32) {
             if (!run(task.x, b, min(b + 32, task.z), vol)) {

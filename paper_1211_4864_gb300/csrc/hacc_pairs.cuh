@@ -40,6 +40,9 @@ struct KArgs {
     const int4 *tasks;
     const int32_t *order;  // task_order: heaviest first
     const int32_t *n_tasks;
+    const int2 *items;       // the dense kernels' work items: task and segment (hacc_hits.cuh)
+    const int32_t *n_items;
+    int seg_pairs;           // pairs of a dense item
     const float4 *origin;  // per cell (leaf) origin, or NULL: chaining-mesh cell c sits at c w
     const float4 *pos;   // sorted (ox, oy, oz, m)
     const float4 *lam;   // sorted (lx, ly, lz, 0), adjoint only
@@ -47,7 +50,7 @@ struct KArgs {
     float *out_x, *out_y, *out_z, *out_m;
     int32_t *counter;    // tasks taken
     int32_t *hit_count;  // mesh lists: the tasks taken by, and the number of, the hit kernel
-    const int32_t *hit_order;  // its tasks, from this slot downwards
+    const int2 *hit_order;     // its tasks, from this slot downwards
     uint32_t *status;
     PairConsts k;
     const uint32_t *mass_varies;  // 0: every mass equal (the equal-mass force paths); NULL: general
@@ -379,12 +382,13 @@ void pair_consts(const hacc_sr_params *p, PairConsts &K)
 // Workspace of the pair calls: the task counter, the adjoints' sorted
 // cotangents (16 B per particle), the symmetric kernels' float64 sums
 // (3 per particle for the force, 3 or 4 for the adjoint), and the split task order
-// (4 B per particle: a task holds at least one).
+// (8 B per particle: a task holds at least one, and is cut into at most as
+// many segments as it holds particles).
 constexpr int SYM_ACC_MAX = 4;
 
 struct ForceWs {
     int32_t *counter;  // the dense and the hit kernel's task counters and task counts
-    int32_t *order;    // the split task order (hacc_hits.cuh), one slot per particle
+    int2 *items;       // the split task order (hacc_hits.cuh), one slot per particle
     float4 *lam;
     double *acc;
     size_t total;
@@ -399,8 +403,8 @@ ForceWs force_layout(const hacc_mesh *mesh, void *ws)
     F.lam = reinterpret_cast<float4 *>(p ? p + 256 : nullptr);
     F.acc = reinterpret_cast<double *>(p ? p + 256 + lam_bytes : nullptr);
     const size_t acc_bytes = round_up((size_t)mesh->N * 8 * SYM_ACC_MAX, 256);
-    F.order = reinterpret_cast<int32_t *>(p ? p + 256 + lam_bytes + acc_bytes : nullptr);
-    F.total = 256 + lam_bytes + acc_bytes + round_up((size_t)mesh->N * 4, 256);
+    F.items = reinterpret_cast<int2 *>(p ? p + 256 + lam_bytes + acc_bytes : nullptr);
+    F.total = 256 + lam_bytes + acc_bytes + round_up((size_t)mesh->N * 8, 256);
     return F;
 }
 

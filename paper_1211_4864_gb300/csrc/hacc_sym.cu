@@ -253,7 +253,7 @@ __device__ __forceinline__ void diag_block_half(const float4 (&oi)[1], bool acti
 // lanes work and each pair is still met once.
 template <int JT, int STAGES, int IPL, bool EQ, bool HALF = false>
 __device__ __forceinline__ bool run_task_sym(const KArgs &a, Ring<FORCE, JT, STAGES> &ring, float *comp, double *acc,
-                                             int64_t N, int lane, int c, int ib, int ie, const hacc_volume &vol)
+                                             int64_t N, int lane, int c, int ib, int ie, const hacc_volume &vol, int code)
 {
     static_assert(!HALF || IPL == 1, "half-warp tasks hold one i set");
     constexpr int W = HALF ? 16 : 32;
@@ -274,16 +274,18 @@ __device__ __forceinline__ bool run_task_sym(const KArgs &a, Ring<FORCE, JT, STA
     }
     AccI<IPL> A(comp, lane);
 
-    // the chunk against itself: block B holds the chunk's i set B as j
-    if constexpr (HALF) {
-        diag_block_half<EQ>(oi, active[0], ib, K, A, acc, N, lane);
-    } else {
-        diag_block<IPL, 0, EQ>(oi, ib, ie, K, A, acc, N, lane);
-    }
-    if constexpr (IPL > 1) diag_block<IPL, 1, EQ>(oi, ib, ie, K, A, acc, N, lane);
-    if constexpr (IPL > 2) {
-        diag_block<IPL, 2, EQ>(oi, ib, ie, K, A, acc, N, lane);
-        diag_block<IPL, 3, EQ>(oi, ib, ie, K, A, acc, N, lane);
+    // the chunk against itself (the task's first segment): block B holds the chunk's i set B as j
+    if ((code & 0xffff) == 0) {
+        if constexpr (HALF) {
+            diag_block_half<EQ>(oi, active[0], ib, K, A, acc, N, lane);
+        } else {
+            diag_block<IPL, 0, EQ>(oi, ib, ie, K, A, acc, N, lane);
+        }
+        if constexpr (IPL > 1) diag_block<IPL, 1, EQ>(oi, ib, ie, K, A, acc, N, lane);
+        if constexpr (IPL > 2) {
+            diag_block<IPL, 2, EQ>(oi, ib, ie, K, A, acc, N, lane);
+            diag_block<IPL, 3, EQ>(oi, ib, ie, K, A, acc, N, lane);
+        }
     }
     A.fold();
 
@@ -291,7 +293,7 @@ __device__ __forceinline__ bool run_task_sym(const KArgs &a, Ring<FORCE, JT, STA
     const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
     const int64_t mid = self_entry(a, c, e0, e1, vol);
     const int ce = a.cell_start[c + 1];
-    for (int64_t g0 = mid; g0 < e1; g0 += 32) {
+    for (int64_t g0 = first_entry(a, e0, mid); g0 < e1; g0 += 32) {
         const int ng = (int)min((int64_t)32, e1 - g0);
         int jb = 0, cnt = 0;
         float Dx = 0.f, Dy = 0.f, Dz = 0.f;
@@ -303,9 +305,12 @@ __device__ __forceinline__ bool run_task_sym(const KArgs &a, Ring<FORCE, JT, STA
                 const int cp = a.nbr_cell[g0 + lane];
                 jb = a.cell_start[cp];
                 cnt = a.cell_start[cp + 1] - jb;
+                if (!takes_entry(g0 + lane, mid, cnt)) cnt = 0;
                 entry_delta(a, vol, cp, a.nbr_shift[g0 + lane], cx, cy, cz, org_i, Dx, Dy, Dz);
             }
         }
+        if (code != SEG_WHOLE)
+            clip_entry(a, lane, code, ie - ib, first_entry(a, e0, mid), mid, g0, jb, cnt, ce - ie);
         int pk = 0, poff = 0;  // producer cursor
         int ck = 0, coff = 0;  // consumer cursor
         for (int s = 0; s < STAGES; ++s)
@@ -390,14 +395,45 @@ __host__ __device__ constexpr int sym_warp_smem_bytes(int jt, int stages)
     return (warp_tiles_bytes(FORCE, jt, stages) + SYM_COMP_BYTES + stages * 8 + 127) / 128 * 128;
 }
 
-// EQ: the equal-mass instantiation.  Both are launched when the binning
-// checked the masses, and the one that does not match the flag returns at
-// once; each keeps its own register allocation.
+// The tasks of one launch, on the equal-mass (EQ) or the general path.
 template <int JT, int STAGES, bool EQ>
+__device__ __forceinline__ void sym_tasks(const KArgs &a, Ring<FORCE, JT, STAGES> &ring, float *comp, double *acc,
+                                          int64_t N, int lane)
+{
+    const int ntask = *a.n_items;
+    while (true) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(a.counter, 1);
+        t = __shfl_sync(FULL, t, 0);
+        if (t >= ntask) break;
+        int4 task;
+        const int2 item = a.items[t];
+        if (!take_task(a, item.x, lane, task)) continue;
+        const hacc_volume &vol = a.vols[task.w];
+        bool ok;
+        const int size = task.z - task.y;
+        if (size > 64)
+            ok = run_task_sym<JT, STAGES, 4, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else if (size > 32)
+            ok = run_task_sym<JT, STAGES, 2, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else if (size > 16)
+            ok = run_task_sym<JT, STAGES, 1, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else
+            ok = run_task_sym<JT, STAGES, 1, EQ, true>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        if (!ok) {
+            if (lane == 0) atomicOr(a.status, HACC_STATUS_TIMEOUT);
+            ring.drain();
+            return;
+        }
+    }
+}
+
+// The two mass paths share the kernel (the device flag picks one), and the
+// hit kernel behind it may start as soon as this one's blocks leave room.
+template <int JT, int STAGES>
 __global__ void __launch_bounds__(256, 3) k_pairs_sym(const KArgs a, double *acc, int64_t N)
 {
-    const bool eq = a.mass_varies && *a.mass_varies == 0u;
-    if (eq != EQ) return;
+    allow_next_kernel();
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int WARP_BYTES = sym_warp_smem_bytes(JT, STAGES);
     constexpr int TILE_BYTES = warp_tiles_bytes(FORCE, JT, STAGES);
@@ -413,31 +449,10 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sym(const KArgs a, double *acc
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
-    const int ntask = task_count(a);
-    while (true) {
-        int t = 0;
-        if (lane == 0) t = atomicAdd(a.counter, 1);
-        t = __shfl_sync(FULL, t, 0);
-        if (t >= ntask) break;
-        int4 task;
-        if (!take_task(a, a.order[t], lane, task)) continue;
-        const hacc_volume &vol = a.vols[task.w];
-        bool ok;
-        const int size = task.z - task.y;
-        if (size > 64)
-            ok = run_task_sym<JT, STAGES, 4, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol);
-        else if (size > 32)
-            ok = run_task_sym<JT, STAGES, 2, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol);
-        else if (size > 16)
-            ok = run_task_sym<JT, STAGES, 1, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol);
-        else
-            ok = run_task_sym<JT, STAGES, 1, EQ, true>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol);
-        if (!ok) {
-            if (lane == 0) atomicOr(a.status, HACC_STATUS_TIMEOUT);
-            ring.drain();
-            return;
-        }
-    }
+    if (a.mass_varies && *a.mass_varies == 0u)
+        sym_tasks<JT, STAGES, true>(a, ring, comp, acc, N, lane);
+    else
+        sym_tasks<JT, STAGES, false>(a, ring, comp, acc, N, lane);
 }
 
 // One component of the float64 totals (sorted slots) to float32 in input
@@ -447,17 +462,19 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sym(const KArgs a, double *acc
 // partial sector is then read and written back in DRAM).  The streamed totals
 // and perm are loaded evict-first for the same reason.
 __global__ void __launch_bounds__(256)
-k_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm, float *__restrict__ out)
+k_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
+             const int32_t *__restrict__ n_dense, float *__restrict__ out)
 {
+    if (no_totals(n_dense)) return;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
         out[__ldcs(perm + k)] = (float)__ldcs(acc + k);
 }
 
-template <int JT, int STAGES, bool EQ>
-int launch_sym_one(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
+template <int JT, int STAGES>
+int launch_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
 {
     const size_t smem = (size_t)warps * sym_warp_smem_bytes(JT, STAGES);
-    auto kern = k_pairs_sym<JT, STAGES, EQ>;
+    auto kern = k_pairs_sym<JT, STAGES>;
     if (smem > 48 * 1024)
         HACC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
@@ -467,16 +484,6 @@ int launch_sym_one(const KArgs &a, double *acc, int64_t N, int warps, int ctas_p
     kern<<<num_sms() * per_sm, warps * 32, smem, st>>>(a, acc, N);
     HACC_LAUNCH_CHECK();
     return HACC_OK;
-}
-
-template <int JT, int STAGES>
-int launch_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
-{
-    if (a.mass_varies) {
-        const int rc = launch_sym_one<JT, STAGES, true>(a, acc, N, warps, ctas_per_sm, st);
-        if (rc) return rc;
-    }
-    return launch_sym_one<JT, STAGES, false>(a, acc, N, warps, ctas_per_sm, st);
 }
 
 int launch_sym(const KArgs &a, double *acc, int64_t N, const hacc_launch &L, cudaStream_t st)
@@ -507,9 +514,14 @@ extern "C" int hacc_sr_force_symmetric(const hacc_mesh *mesh, const hacc_binned 
     cudaStream_t st = as_stream(stream);
     ForceWs F = force_layout(mesh, ws);
     KArgs a = base_args(mesh, binned, lists, p, status);
-    a.counter = F.counter;
-    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
-    HACC_CUDA_TRY(cudaMemsetAsync(F.acc, 0, (size_t)mesh->N * 3 * sizeof(double), st));
+    a.out_x = ax;
+    a.out_y = ay;
+    a.out_z = az;
+    rc = split_tasks(a, F, false, st);
+    if (rc) return rc;
+    const int32_t *n_dense = a.n_items;
+    rc = zero_totals(a, F.acc, 3, n_dense, st);
+    if (rc) return rc;
     hacc_launch L;
     if (launch) {
         L = *launch;
@@ -523,11 +535,15 @@ extern "C" int hacc_sr_force_symmetric(const hacc_mesh *mesh, const hacc_binned 
     a.wait_limit = wait_limit_of(L);
     rc = launch_sym(a, F.acc, mesh->N, L, st);
     if (rc) return rc;
+    if (!a.origin) {
+        rc = launch_hits(k_hits_sym<FORCE>, FORCE, st, a, F.acc);
+        if (rc) return rc;
+    }
     int g = (int)((mesh->N + 255) / 256);
     if (g > num_sms() * 16) g = num_sms() * 16;
     float *out[3] = {ax, ay, az};
     for (int c = 0; c < 3; ++c) {
-        k_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, out[c]);
+        k_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, n_dense, out[c]);
         HACC_LAUNCH_CHECK();
     }
     return HACC_OK;

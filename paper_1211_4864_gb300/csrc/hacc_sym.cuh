@@ -3,30 +3,13 @@
 // of a cell itself and the image offset of a list entry.
 #pragma once
 
-#include "hacc_pairs.cuh"
+#include "hacc_hits.cuh"
 
 namespace hacc {
 namespace {
 
 // Position of an empty lane: every pair with it fails the cutoff test.
 constexpr float FAR = 1.0e6f;
-
-// The list entry of cell (or leaf) c itself, image 13.  A chaining-mesh list
-// is symmetric under d -> -d with the cell in the middle; a tree leaf's list
-// is sorted by (image code, leaf id) and symmetric too (leaf j with image s
-// is listed for i iff i with image -s is listed for j), so its own entry is
-// found by bisection and everything after it is the forward half.
-__device__ __forceinline__ int64_t self_entry(const KArgs &a, int c, int64_t e0, int64_t e1, const hacc_volume &vol)
-{
-    if (!a.origin) return e0 + (vol.S - 1) / 2;
-    int64_t lo = e0, hi = e1 - 1;
-    while (lo < hi) {  // first entry with (code, leaf) >= (13, c)
-        const int64_t mid = (lo + hi) >> 1;
-        const int code = a.nbr_shift[mid], leaf = a.nbr_cell[mid];
-        if (code < 13 || (code == 13 && leaf < c)) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
 
 // Image offset Delta of one list entry: origin of cell (leaf) cp shifted by
 // the image, minus the origin of c; float64, rounded once.
@@ -50,6 +33,96 @@ __device__ __forceinline__ void entry_delta(const KArgs &a, const hacc_volume &v
         Dy = (float)((double)cell_centre(py, w) - (double)cell_centre(cy, w) + sy * Ld);
         Dz = (float)((double)cell_centre(pz, w) - (double)cell_centre(cz, w) + sz * Ld);
     }
+}
+
+// Lane's entry of the group at g0 (first record jb, cnt of them) clipped to
+// the segment's j records of the task's flattened list, whose entries start at
+// e_first.  size: the task's particles.
+__device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, int size, int64_t e_first, int64_t mid,
+                                           int64_t g0, int &jb, int &cnt, int own)
+{
+    int before = 0;  // records of the groups before (lists of more than 32 entries)
+    for (int64_t e = e_first + lane; e < g0; e += 32) {
+        int n = own;
+        if (e != mid) {
+            n = a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
+            if (!takes_entry(e, mid, n)) n = 0;
+        }
+        before += n;
+    }
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += t;
+    }
+    const int per = segment_records(a, size) << ((code >> 16) & 31), jlo = (code & 0xffff) * per;
+    const int first = (int)__reduce_add_sync(FULL, (unsigned)before) + inc - cnt;
+    const int lo = max(first, jlo), hi = code >> 24 ? first + cnt : min(first + cnt, jlo + per);
+    jb += lo - first;
+    cnt = max(hi - lo, 0);
+}
+
+// Without dense tasks (n_dense given and 0) the hit kernel stores every
+// output itself: the totals are then neither zeroed nor converted.
+__device__ __forceinline__ bool no_totals(const int32_t *n_dense) { return n_dense && *n_dense == 0; }
+
+__global__ void __launch_bounds__(256)
+k_zero_totals(double2 *__restrict__ acc, int64_t n2, const int32_t *__restrict__ n_dense)
+{
+    if (no_totals(n_dense)) return;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n2; k += (int64_t)gridDim.x * blockDim.x)
+        acc[k] = make_double2(0.0, 0.0);
+}
+
+// Zeroes nc totals per particle (the region holds SYM_ACC_MAX of them).
+int zero_totals(const KArgs &a, double *acc, int nc, const int32_t *n_dense, cudaStream_t st)
+{
+    const int64_t n2 = (a.N * nc + 1) / 2;
+    int64_t g = (n2 + 255) / 256;
+    if (g > num_sms() * 16) g = num_sms() * 16;
+    k_zero_totals<<<(int)g, 256, 0, st>>>(reinterpret_cast<double2 *>(acc), n2, n_dense);
+    HACC_LAUNCH_CHECK();
+    return HACC_OK;
+}
+
+// One hit-mask task of a symmetric call (the small cells' pairs): its totals
+// are stored (no dense tasks) or added to the float64 totals, to which dense
+// tasks add the pairs with their cells.
+template <int MODE>
+__device__ __forceinline__ bool hit_task_sym(const KArgs &a, HitWarp &W, int lane, int c, int ib, int ie,
+                                             const hacc_volume &vol, double *acc, bool eq, bool store)
+{
+    HitAcc<MODE> A;
+    float4 oi, li;
+    int i;
+    bool active;
+    if (!run_hits<MODE>(a, W.base, W.bar, W.phase, lane, c, ib, ie, vol, eq, true, A, oi, li, i, active))
+        return false;
+    if (!active) return true;
+    if (store) {
+        store_out<MODE>(a, a.perm[i], oi, eq, [&](int k) { return A.total(k); });
+    } else {
+        // the force's totals hold the mass, the adjoint's are scaled by the finishing pass
+        const double m = MODE == FORCE && eq ? (double)oi.w : 1.0;
+#pragma unroll
+        for (int k = 0; k < HitAcc<MODE>::NC; ++k)
+            atomicAdd(acc + k * a.N + i, m * ((double)A.h[k] + (double)A.l[k]));
+    }
+    return true;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(HITS_WARPS * 32, hits_ctas(MODE)) k_hits_sym(const KArgs a, double *acc)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    HitWarp W = hits_warp(smem, warp, lane, MODE);
+    const bool eq = a.mass_varies && *a.mass_varies == 0u, store = no_totals(a.n_items);
+    hits_tasks(a, lane, [&](int c, int ib, int ie, const hacc_volume &vol) {
+        return hit_task_sym<MODE>(a, W, lane, c, ib, ie, vol, acc, eq, store);
+    });
+    wait_previous_kernel();
 }
 
 }  // namespace

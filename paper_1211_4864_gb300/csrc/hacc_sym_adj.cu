@@ -142,7 +142,7 @@ __device__ __forceinline__ void own_block_adj(const float4 (&oi)[IPL], const flo
 template <int JT, int STAGES, int IPL, bool GM, bool EQ, bool HALF = false>
 __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, JT, STAGES> &ring, float *comp,
                                                  double *acc, int64_t N, int lane, int c, int ib, int ie,
-                                                 const hacc_volume &vol)
+                                                 const hacc_volume &vol, int code)
 {
     static_assert(!HALF || IPL == 1, "half-warp tasks hold one i set");
     constexpr int W = HALF ? 16 : 32;
@@ -165,31 +165,33 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
     }
     AccAdj<MODE, IPL, adj_nacc(MODE)> A(comp, lane);
 
-    if constexpr (HALF) {  // the chunk against itself on the low half-warp, 16 steps
-        const bool lo = lane < 16;
-        JAdj J{oi[0].x, oi[0].y, oi[0].z, oi[0].w, li[0].x, li[0].y, li[0].z,
-               0.f, 0.f, 0.f, 0.f, (lo && active[0]) ? ib + lane : -1};
-        if (!lo) {
-            J.x = J.y = J.z = FAR;
-            J.m = J.lx = J.ly = J.lz = 0.f;
+    if ((code & 0xffff) == 0) {  // the task's first segment
+        if constexpr (HALF) {  // the chunk against itself on the low half-warp, 16 steps
+            const bool lo = lane < 16;
+            JAdj J{oi[0].x, oi[0].y, oi[0].z, oi[0].w, li[0].x, li[0].y, li[0].z,
+                   0.f, 0.f, 0.f, 0.f, (lo && active[0]) ? ib + lane : -1};
+            if (!lo) {
+                J.x = J.y = J.z = FAR;
+                J.m = J.lx = J.ly = J.lz = 0.f;
+            }
+            rotate_block_adj<1, GM, EQ, 1u, 0u, 16>(J, oi, li, K, A.p, lane);
+            flush_adj<GM, EQ>(J, acc, N);
+            A.fold();
+        } else {  // the chunk against itself
+            own_block_adj<0, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
+            if constexpr (IPL >= 2) own_block_adj<1, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
+            if constexpr (IPL >= 4) {
+                own_block_adj<2, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
+                own_block_adj<3, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
+            }
+            A.fold();
         }
-        rotate_block_adj<1, GM, EQ, 1u, 0u, 16>(J, oi, li, K, A.p, lane);
-        flush_adj<GM, EQ>(J, acc, N);
-        A.fold();
-    } else {  // the chunk against itself
-        own_block_adj<0, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
-        if constexpr (IPL >= 2) own_block_adj<1, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
-        if constexpr (IPL >= 4) {
-            own_block_adj<2, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
-            own_block_adj<3, IPL, GM, EQ>(oi, li, active, ib, lane, K, A.p, acc, N);
-        }
-        A.fold();
     }
 
     const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
     const int64_t mid = self_entry(a, c, e0, e1, vol);
     const int ce = a.cell_start[c + 1];
-    for (int64_t g0 = mid; g0 < e1; g0 += 32) {
+    for (int64_t g0 = first_entry(a, e0, mid); g0 < e1; g0 += 32) {
         const int ng = (int)min((int64_t)32, e1 - g0);
         int jb = 0, cnt = 0;
         float Dx = 0.f, Dy = 0.f, Dz = 0.f;
@@ -201,9 +203,12 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
                 const int cp = a.nbr_cell[g0 + lane];
                 jb = a.cell_start[cp];
                 cnt = a.cell_start[cp + 1] - jb;
+                if (!takes_entry(g0 + lane, mid, cnt)) cnt = 0;
                 entry_delta(a, vol, cp, a.nbr_shift[g0 + lane], cx, cy, cz, org_i, Dx, Dy, Dz);
             }
         }
+        if (code != SEG_WHOLE)
+            clip_entry(a, lane, code, ie - ib, first_entry(a, e0, mid), mid, g0, jb, cnt, ce - ie);
         int pk = 0, poff = 0;
         int ck = 0, coff = 0;
         for (int s = 0; s < STAGES; ++s)
@@ -275,11 +280,45 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
     return true;
 }
 
+// The tasks of one launch, on the equal-mass (EQ) or the general path.
 template <int JT, int STAGES, bool GM, bool EQ>
+__device__ __forceinline__ void adj_sym_tasks(const KArgs &a, Ring<ADJOINT, JT, STAGES> &ring, float *comp,
+                                              double *acc, int64_t N, int lane)
+{
+    const int ntask = *a.n_items;
+    while (true) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(a.counter, 1);
+        t = __shfl_sync(FULL, t, 0);
+        if (t >= ntask) break;
+        int4 task;
+        const int2 item = a.items[t];
+        if (!take_task(a, item.x, lane, task)) continue;
+        const hacc_volume &vol = a.vols[task.w];
+        bool ok;
+        const int size = task.z - task.y;
+        if (size > 64)
+            ok = run_task_adj_sym<JT, STAGES, 4, GM, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else if (size > 32)
+            ok = run_task_adj_sym<JT, STAGES, 2, GM, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else if (size > 16)
+            ok = run_task_adj_sym<JT, STAGES, 1, GM, EQ>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol, item.y);
+        else
+            ok = run_task_adj_sym<JT, STAGES, 1, GM, EQ, true>(a, ring, comp, acc, N, lane, task.x, task.y, task.z, vol,
+                                                               item.y);
+        if (!ok) {
+            if (lane == 0) atomicOr(a.status, HACC_STATUS_TIMEOUT);
+            ring.drain();
+            return;
+        }
+    }
+}
+
+// The two mass paths share the kernel, as the force's (k_pairs_sym).
+template <int JT, int STAGES, bool GM>
 __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, int64_t N)
 {
-    const bool eq = a.mass_varies && *a.mass_varies == 0u;
-    if (eq != EQ) return;  // the other instantiation does the work
+    allow_next_kernel();
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int WARP_BYTES = warp_smem_bytes(ADJOINT, JT, STAGES);
     constexpr int TILE_BYTES = warp_tiles_bytes(ADJOINT, JT, STAGES);
@@ -295,36 +334,10 @@ __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, 
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
-    const int ntask = task_count(a);
-    while (true) {
-        int t = 0;
-        if (lane == 0) t = atomicAdd(a.counter, 1);
-        t = __shfl_sync(FULL, t, 0);
-        if (t >= ntask) break;
-        int4 task;
-        if (!take_task(a, a.order[t], lane, task)) continue;
-        const hacc_volume &vol = a.vols[task.w];
-        bool ok = true;
-        // larger tasks: four i per lane, chunks of 128 particles
-        constexpr int CHUNK = 128;
-        for (int sb = task.y; ok && sb < task.z; sb += CHUNK) {
-            const int se = min(sb + CHUNK, task.z);
-            if (se - sb > 64)
-                ok = run_task_adj_sym<JT, STAGES, 4, GM, EQ>(a, ring, comp, acc, N, lane, task.x, sb, se, vol);
-            else if (se - sb > 32)
-                ok = run_task_adj_sym<JT, STAGES, 2, GM, EQ>(a, ring, comp, acc, N, lane, task.x, sb, se, vol);
-            else if (se - sb > 16)
-                ok = run_task_adj_sym<JT, STAGES, 1, GM, EQ>(a, ring, comp, acc, N, lane, task.x, sb, se, vol);
-            else
-                ok = run_task_adj_sym<JT, STAGES, 1, GM, EQ, true>(a, ring, comp, acc, N, lane, task.x, sb, se,
-                                                                   vol);
-        }
-        if (!ok) {
-            if (lane == 0) atomicOr(a.status, HACC_STATUS_TIMEOUT);
-            ring.drain();
-            return;
-        }
-    }
+    if (a.mass_varies && *a.mass_varies == 0u)
+        adj_sym_tasks<JT, STAGES, GM, true>(a, ring, comp, acc, N, lane);
+    else
+        adj_sym_tasks<JT, STAGES, GM, false>(a, ring, comp, acc, N, lane);
 }
 
 // One output component from its float64 totals, in input order: dL/dx = W
@@ -333,19 +346,20 @@ __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, 
 __global__ void __launch_bounds__(256)
 k_adj_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
                  const float4 *__restrict__ pos, const uint32_t *mass_varies, bool is_gm,
-                 float *__restrict__ out)
+                 const int32_t *__restrict__ n_dense, float *__restrict__ out)
 {
+    if (no_totals(n_dense)) return;
     const bool eq = mass_varies && *mass_varies == 0u;
     const double sc = is_gm ? -1.0 : eq ? (double)pos[0].w : 1.0;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
         out[__ldcs(perm + k)] = (float)(sc * __ldcs(acc + k));
 }
 
-template <int JT, int STAGES, bool GM, bool EQ>
-int launch_adj_sym_one(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
+template <int JT, int STAGES, bool GM>
+int launch_adj_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
 {
     const size_t smem = (size_t)warps * warp_smem_bytes(ADJOINT, JT, STAGES);
-    auto kern = k_adj_sym<JT, STAGES, GM, EQ>;
+    auto kern = k_adj_sym<JT, STAGES, GM>;
     if (smem > 48 * 1024)
         HACC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
@@ -355,16 +369,6 @@ int launch_adj_sym_one(const KArgs &a, double *acc, int64_t N, int warps, int ct
     kern<<<num_sms() * per_sm, warps * 32, smem, st>>>(a, acc, N);
     HACC_LAUNCH_CHECK();
     return HACC_OK;
-}
-
-template <int JT, int STAGES, bool GM>
-int launch_adj_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
-{
-    if (a.mass_varies) {
-        const int rc = launch_adj_sym_one<JT, STAGES, GM, true>(a, acc, N, warps, ctas_per_sm, st);
-        if (rc) return rc;
-    }
-    return launch_adj_sym_one<JT, STAGES, GM, false>(a, acc, N, warps, ctas_per_sm, st);
 }
 
 template <bool GM>
@@ -402,9 +406,15 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
     HACC_LAUNCH_CHECK();
     KArgs a = base_args(mesh, binned, lists, p, status);
     a.lam = F.lam;
-    a.counter = F.counter;
-    HACC_CUDA_TRY(cudaMemsetAsync(F.counter, 0, sizeof(int32_t), st));
-    HACC_CUDA_TRY(cudaMemsetAsync(F.acc, 0, (size_t)mesh->N * (gm ? 4 : 3) * sizeof(double), st));
+    a.out_x = gx;
+    a.out_y = gy;
+    a.out_z = gz;
+    a.out_m = gm;
+    rc = split_tasks(a, F, false, st);
+    if (rc) return rc;
+    const int32_t *n_dense = a.n_items;
+    rc = zero_totals(a, F.acc, gm ? 4 : 3, n_dense, st);
+    if (rc) return rc;
     hacc_launch L;
     if (launch) {
         L = *launch;
@@ -418,11 +428,16 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
     a.wait_limit = wait_limit_of(L);
     rc = gm ? launch_adj_sym<true>(a, F.acc, mesh->N, L, st) : launch_adj_sym<false>(a, F.acc, mesh->N, L, st);
     if (rc) return rc;
+    if (!a.origin) {
+        rc = gm ? launch_hits(k_hits_sym<ADJOINT_GM>, ADJOINT_GM, st, a, F.acc)
+                : launch_hits(k_hits_sym<ADJOINT>, ADJOINT, st, a, F.acc);
+        if (rc) return rc;
+    }
     const float4 *pos = reinterpret_cast<const float4 *>(binned->sorted4);
     float *out[4] = {gx, gy, gz, gm};
     for (int c = 0; c < (gm ? 4 : 3); ++c) {
         k_adj_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, pos, binned->mass_varies,
-                                            c == 3, out[c]);
+                                            c == 3, n_dense, out[c]);
         HACC_LAUNCH_CHECK();
     }
     return HACC_OK;

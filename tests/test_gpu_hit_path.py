@@ -1,9 +1,10 @@
 """The hit path of the pair kernels (chaining-mesh cells of few particles).
 
 Cells of n particles each at the edges of its row tiles (8, 16, 32), of the
-cell size it takes (64 and 65) and of its batches of 256 candidates (27 cells
+cell size it takes (40 and 41) and of its batches of 256 candidates (27 cells
 of 9 and 10, a last step of one record), small cells around one large cell
-(both kernels add to the same particles), and a fine mesh whose lists span
+(both kernels add to the same particles; the largest is cut into segments),
+and a fine mesh whose lists span
 several groups of 32 entries.  Every pair call on both mass paths against the
 float64 oracle; the gather calls again bit for bit."""
 
@@ -48,7 +49,7 @@ def rounding_bounds(pos, m, lam, L):
 
 CASES = [(1, 3, 0, 3.0, 32), (8, 3, 0, 3.0, 32), (9, 3, 0, 3.0, 32), (10, 4, 0, 3.0, 64), (16, 3, 0, 3.0, 32),
          (17, 3, 0, 3.0, 32), (32, 3, 0, 3.0, 32), (33, 3, 0, 3.0, 32), (33, 3, 0, 3.0, 64), (64, 3, 0, 3.0, 128),
-         (65, 3, 0, 3.0, 128), (12, 3, 300, 3.0, 128), (20, 3, 70, 3.0, 32), (19, 4, 0, 1.5, 32), (3, 3, 0, 0.75, 32)]
+         (65, 3, 0, 3.0, 128), (40, 3, 0, 3.0, 64), (41, 3, 0, 3.0, 64), (12, 3, 300, 3.0, 128), (20, 3, 70, 3.0, 32), (12, 3, 2000, 3.0, 128), (19, 4, 0, 1.5, 32), (3, 3, 0, 0.75, 32)]
 
 
 @pytest.mark.parametrize("n,side,big,cell_min,split_T", CASES)
