@@ -5,7 +5,8 @@ One step = the whole hot path on one synthetic workload resident in HBM:
 chaining-mesh binning -> neighbour lists and tasks -> pair force -> kick ->
 float64 moments (momentum, Newton-III residual, kinetic energy).  The metric
 is candidate pair interactions per second (the ordered pairs j != i that the
-force kernel evaluates, counted by the list builder), whole job over all
+lists hold and the step decides, counted by the list builder; cells of few
+particles evaluate only those near or inside the cutoff), whole job over all
 ranks.  Default workload: 256^3 = 16,777,216 particles, 60 % uniform and 40 %
 in 2000 NFW halos, box 256, r_c = 3, eps = 0.01 (the clustered configuration
 the throughput target is stated on).
@@ -42,10 +43,10 @@ FLOPS_PER_SYM_PAIR_EQ = 34  # equal-mass path: no x m_j, x m_i
 # were taken from (null in the bench line once a source changes)
 FORCE_TRAFFIC = {
     "gather": {"workload": "clustered256", "bytes": 2215769856 + 965738240,
-               "sources": ["hacc_force.cu", "hacc_pairs.cuh", "hacc_common.cuh"],
+               "sources": ["hacc_force.cu", "hacc_hits.cuh", "hacc_terms.cuh", "hacc_pairs.cuh", "hacc_common.cuh"],
                "sha256": "f33c028c24cff617ab446f124bf0640bec48672f709b34739964367f8e5d7fe2"},
     "symmetric": {"workload": "clustered256", "bytes": 2792809216 + 1489363968,
-                  "sources": ["hacc_sym.cu", "hacc_sym.cuh", "hacc_pairs.cuh", "hacc_common.cuh"],
+                  "sources": ["hacc_sym.cu", "hacc_sym.cuh", "hacc_hits.cuh", "hacc_pairs.cuh", "hacc_common.cuh"],
                   "sha256": "2f782f4823a30586354eecabd2d1f6a1934ce8370423d01b11480201df88b556"},
 }
 METRIC = "short-range pair interactions/s"
@@ -333,16 +334,17 @@ def run_ours(args):
         pass
     f_max = float(peaks.get("sm_max_mhz", 2070.0))
     peak = sms * 128 * 2 * f_max * 1e6 / 1e12
-    # the roofline's numerator: the flops the kernel executes per evaluated pair times the pairs it
-    # evaluates in one launch.  The gather kernel evaluates every ordered candidate pair; the
-    # symmetric kernel evaluates each unordered pair once and applies it to both particles, so it
-    # evaluates half the interactions the step covers (with both accumulations in its flop count).
+    # the roofline's numerator: the flops per evaluated pair times the pairs inside the cutoff.  The
+    # dense kernels evaluate every candidate, the hit kernels (cells of few particles) little more
+    # than the pairs inside the cutoff, so this counts what every path has to evaluate and no
+    # rejected candidate.  The symmetric kernel evaluates each unordered pair once and applies it to
+    # both particles (both accumulations in its flop count).
     if args.kernel == "symmetric":
-        evaluated = pairs // 2
+        evaluated = within // 2
         fpp = fpp_s
         kname = "k_pairs_sym (hacc_sr_force_symmetric)"
     else:
-        evaluated = pairs
+        evaluated = within
         fpp = fpp_g
         kname = "k_pairs<FORCE> (hacc_sr_force)"
     achieved = fpp * evaluated / (t_force * 1e-3) / 1e12
@@ -350,7 +352,7 @@ def run_ours(args):
     out["roofline"] = {"bound": "alu", "kernel": kname, "achieved": achieved,
                        "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                        "traffic": force_traffic(args.config, args.kernel),
-                       "flops_per_evaluated_pair": fpp, "evaluated_pairs_per_launch": evaluated,
+                       "flops_per_evaluated_pair": fpp, "pairs_within_cutoff_counted": evaluated,
                        "interactions_per_launch": pairs,
                        "mass_path": "equal (every particle mass equal)" if eq else "general (per-particle masses)",
                        "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 x {f_max:.0f} MHz (max SM clock)",
@@ -366,7 +368,7 @@ def run_ours(args):
     # the other pair kernel on the same lists: Newton-III symmetric vs gather
     if ranks.rank == 0:
         out["newton3"] = newton3(torch, sr, prm, launch, launch_sym, a, pairs, args.kernel, t_force, peak,
-                                 fpp_g, fpp_s)
+                                 fpp_g, fpp_s, within)
 
     # forward + adjoint on the same lists (not part of the timed step)
     lam = torch.randn((3, w.N), device=dev, generator=torch.Generator(device=dev).manual_seed(7))
@@ -558,7 +560,7 @@ def binning_rate(torch, sr, pos, m, w, peaks, reps=5):
                     "intermediate reads and writes are not counted as algorithmic bytes"}
 
 
-def newton3(torch, sr, prm, launch, launch_sym, a, pairs, kernel, t_force, peak, fpp_g, fpp_s, reps=3):
+def newton3(torch, sr, prm, launch, launch_sym, a, pairs, kernel, t_force, peak, fpp_g, fpp_s, within, reps=3):
     """Gather kernel (every particle sums its own list: each pair evaluated
     twice) against the Newton-III symmetric kernel (each pair once, applied to
     both), same lists, same inputs; the one the step did not use is timed
@@ -580,8 +582,8 @@ def newton3(torch, sr, prm, launch, launch_sym, a, pairs, kernel, t_force, peak,
     rel = float((a.double() - b.double()).norm() / b.double().norm())
     return {"gather_force_ms": t_g, "symmetric_force_ms": t_s, "speedup": t_g / t_s,
             "interactions_per_s": {"gather": pairs / (t_g * 1e-3), "symmetric": pairs / (t_s * 1e-3)},
-            "fp32_frac": {"gather": fpp_g * pairs / (t_g * 1e-3) / 1e12 / peak,
-                          "symmetric": fpp_s * (pairs // 2) / (t_s * 1e-3) / 1e12 / peak},
+            "fp32_frac": {"gather": fpp_g * within / (t_g * 1e-3) / 1e12 / peak,
+                          "symmetric": fpp_s * (within // 2) / (t_s * 1e-3) / 1e12 / peak},
             "force_rel_diff": rel,
             "launch": {"gather": launch.__dict__ if launch else "default",
                        "symmetric": launch_sym.__dict__ if launch_sym else "default"}}
@@ -618,9 +620,10 @@ def mass_paths(torch, sr, pos, m, prm, lam, launches, a, pairs, peak, eq_ms, rep
     sr.set_equal_mass_path(True)
     sr.prepare(pos, m)
     torch.cuda.synchronize()
+    within = sr.pairs_within_cutoff(prm)
     t["fp32_frac"] = {
-        "gather": FLOPS_PER_PAIR * pairs / (t["gather_force_ms"] * 1e-3) / 1e12 / peak,
-        "symmetric": FLOPS_PER_SYM_PAIR * (pairs // 2) / (t["symmetric_force_ms"] * 1e-3) / 1e12 / peak}
+        "gather": FLOPS_PER_PAIR * within / (t["gather_force_ms"] * 1e-3) / 1e12 / peak,
+        "symmetric": FLOPS_PER_SYM_PAIR * (within // 2) / (t["symmetric_force_ms"] * 1e-3) / 1e12 / peak}
     return {"general": t,
             "equal_mass_speedup": {k: t[k] / eq_ms[k] for k in eq_ms},
             "force_rel_diff_equal_vs_general": rel}
@@ -957,11 +960,12 @@ def sweep(args):
             sr.prepare(pos, m)
             torch.cuda.synchronize()
             pairs = sr.pair_count()
+            within = sr.pairs_within_cutoff(prm)
             eq = sr.equal_mass  # unit masses: the equal-mass path, and its executed flops
             out = torch.empty((3, n), device="cuda")
-            for kernel, fn, flops in (("gather", sr.force, (FLOPS_PER_PAIR_EQ if eq else FLOPS_PER_PAIR) * pairs),
+            for kernel, fn, flops in (("gather", sr.force, (FLOPS_PER_PAIR_EQ if eq else FLOPS_PER_PAIR) * within),
                                       ("symmetric", sr.force_symmetric,
-                                       (FLOPS_PER_SYM_PAIR_EQ if eq else FLOPS_PER_SYM_PAIR) * pairs / 2)):
+                                       (FLOPS_PER_SYM_PAIR_EQ if eq else FLOPS_PER_SYM_PAIR) * within / 2)):
                 for cps in (1, 2, 3):
                     L = hs.Launch(8, cps, 128, 2)
                     fn(prm, out, launch=L)
