@@ -138,7 +138,9 @@ typedef struct hacc_sr_params {
 } hacc_sr_params;
 
 /* Launch shape of the pair kernels (host struct; NULL = built-in default).
- * The autotuner picks these per workload. */
+ * The autotuner picks these per workload.  Chaining-mesh cells of few
+ * particles run in a kernel of its own fixed shape, to which only wait_cycles
+ * applies. */
 typedef struct hacc_launch {
     int32_t warps_per_cta; /* 1..8 */
     int32_t ctas_per_sm;   /* resident CTAs per SM of the persistent grid, 1..8 */
@@ -319,7 +321,7 @@ size_t hacc_rcb_lists_workspace_size(const hacc_mesh *mesh, int64_t leaf_cap, in
 int hacc_rcb_lists(const hacc_mesh *mesh, const hacc_tree *tree, const hacc_lists *lists, int64_t entry_cap,
                    int64_t *n_entries, void *ws, size_t ws_bytes, uint32_t *status, void *stream);
 
-/* Bytes of scratch that hacc_sr_force / hacc_sr_force_adjoint need. */
+/* Bytes of scratch that each force, adjoint and potential call needs. */
 size_t hacc_force_workspace_size(const hacc_mesh *mesh);
 
 /* Short-range force (Eq. 7) on every particle, written to ax, ay, az [N] in

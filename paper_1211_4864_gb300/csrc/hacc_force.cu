@@ -8,7 +8,8 @@
 // (cp.async.bulk, completion on an mbarrier), and each staged j is broadcast to
 // all 32 lanes by a 16-byte shared load.  Warps take tasks from an atomic
 // counter (a persistent, work-stealing grid), so the very uneven lists of
-// clustered particles balance themselves.
+// clustered particles balance themselves.  Small chaining-mesh cells take the
+// hit path instead (hacc_hits.cuh).
 //
 // Arithmetic per pair (float32, cutoff as a select, as in the paper's
 // branch-free kernel, Sec. III):

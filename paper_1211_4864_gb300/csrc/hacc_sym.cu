@@ -6,7 +6,10 @@
 // Work decomposition.  The same tasks, lists and staging ring as the gather
 // kernel, but each task walks half of its cell's list: the cell itself and
 // the entries after it (lists are symmetric, so every other neighbour pair is
-// met from the other cell); chaining-mesh cells and tree leaves alike.
+// met from the other cell); chaining-mesh cells and tree leaves alike.  Small
+// chaining-mesh cells take the hit path (hacc_hits.cuh) among themselves; the
+// tasks here meet the small cells before theirs too.  A task of many pairs is
+// cut into segments of its j records (hacc_hits.cuh).
 // Inside the cell a task meets its own chunk (pairs j > i) and the particles
 // after the chunk.
 //
@@ -455,21 +458,6 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sym(const KArgs a, double *acc
         sym_tasks<JT, STAGES, false>(a, ring, comp, acc, N, lane);
 }
 
-// One component of the float64 totals (sorted slots) to float32 in input
-// order.  The stores scatter through the permutation, 4 bytes each; they merge
-// into whole sectors in L2 only while the target array stays resident there,
-// which one 67 MB component per launch does and three at once do not (each
-// partial sector is then read and written back in DRAM).  The streamed totals
-// and perm are loaded evict-first for the same reason.
-__global__ void __launch_bounds__(256)
-k_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
-             const int32_t *__restrict__ n_dense, float *__restrict__ out)
-{
-    if (no_totals(n_dense)) return;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-        out[__ldcs(perm + k)] = (float)__ldcs(acc + k);
-}
-
 template <int JT, int STAGES>
 int launch_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
 {
@@ -539,12 +527,6 @@ extern "C" int hacc_sr_force_symmetric(const hacc_mesh *mesh, const hacc_binned 
         rc = launch_hits(k_hits_sym<FORCE>, FORCE, st, a, F.acc);
         if (rc) return rc;
     }
-    int g = (int)((mesh->N + 255) / 256);
-    if (g > num_sms() * 16) g = num_sms() * 16;
-    float *out[3] = {ax, ay, az};
-    for (int c = 0; c < 3; ++c) {
-        k_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, n_dense, out[c]);
-        HACC_LAUNCH_CHECK();
-    }
-    return HACC_OK;
+    float *const out[4] = {ax, ay, az, nullptr};
+    return finish_totals(a, F.acc, n_dense, out, 3, nullptr, st);
 }

@@ -86,6 +86,48 @@ int zero_totals(const KArgs &a, double *acc, int nc, const int32_t *n_dense, cud
     return HACC_OK;
 }
 
+// Output components [c0, c1) from their float64 totals (sorted slots), float32
+// in input order; the adjoints' dL/dx = W times the common mass when the masses
+// are equal (mass_varies given and 0), and their component 3, dL/dm = -G.
+// The stores scatter through the permutation, 4 bytes each; they merge into
+// whole sectors in L2 only while the target array stays resident there, which
+// one 67 MB component of 16.8M particles per launch does and three at once do
+// not (each partial sector is then read and written back in DRAM: 0.82 against
+// 0.33 ms).  The streamed totals and perm are loaded evict-first for the same
+// reason.
+struct TotalsOut {
+    float *out[4];
+};
+__global__ void __launch_bounds__(256)
+k_finish_totals(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
+                const float4 *__restrict__ pos, const uint32_t *mass_varies,
+                const int32_t *__restrict__ n_dense, TotalsOut o, int c0, int c1)
+{
+    if (no_totals(n_dense)) return;
+    const double w = mass_varies && *mass_varies == 0u ? (double)pos[0].w : 1.0;
+    for (int c = c0; c < c1; ++c) {
+        const double sc = c == 3 ? -1.0 : w;
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
+            o.out[c][__ldcs(perm + k)] = (float)(sc * __ldcs(acc + c * N + k));
+    }
+}
+
+// One launch for all components while they fit the L2 together (4M particles:
+// 67 MB), else one each.
+int finish_totals(const KArgs &a, const double *acc, const int32_t *n_dense, float *const (&out)[4], int nc,
+                  const uint32_t *mass_varies, cudaStream_t st)
+{
+    int64_t g = (a.N + 255) / 256;
+    if (g > num_sms() * 16) g = num_sms() * 16;
+    const TotalsOut o{{out[0], out[1], out[2], out[3]}};
+    const int step = a.N <= ((int64_t)4 << 20) ? nc : 1;
+    for (int c = 0; c < nc; c += step) {
+        k_finish_totals<<<(int)g, 256, 0, st>>>(a.N, acc, a.perm, a.pos, mass_varies, n_dense, o, c, c + step);
+        HACC_LAUNCH_CHECK();
+    }
+    return HACC_OK;
+}
+
 // One hit-mask task of a symmetric call (the small cells' pairs): its totals
 // are stored (no dense tasks) or added to the float64 totals, to which dense
 // tasks add the pairs with their cells.

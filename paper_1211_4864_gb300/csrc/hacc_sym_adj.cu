@@ -340,21 +340,6 @@ __global__ void __launch_bounds__(256, 2) k_adj_sym(const KArgs a, double *acc, 
         adj_sym_tasks<JT, STAGES, GM, false>(a, ring, comp, acc, N, lane);
 }
 
-// One output component from its float64 totals, in input order: dL/dx = W
-// (equal masses: m W, m the common mass), dL/dm = -G (is_gm); one
-// component per launch for the reason given at k_sym_finish.
-__global__ void __launch_bounds__(256)
-k_adj_sym_finish(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
-                 const float4 *__restrict__ pos, const uint32_t *mass_varies, bool is_gm,
-                 const int32_t *__restrict__ n_dense, float *__restrict__ out)
-{
-    if (no_totals(n_dense)) return;
-    const bool eq = mass_varies && *mass_varies == 0u;
-    const double sc = is_gm ? -1.0 : eq ? (double)pos[0].w : 1.0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x)
-        out[__ldcs(perm + k)] = (float)(sc * __ldcs(acc + k));
-}
-
 template <int JT, int STAGES, bool GM>
 int launch_adj_sym_t(const KArgs &a, double *acc, int64_t N, int warps, int ctas_per_sm, cudaStream_t st)
 {
@@ -433,12 +418,6 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
                 : launch_hits(k_hits_sym<ADJOINT>, ADJOINT, st, a, F.acc);
         if (rc) return rc;
     }
-    const float4 *pos = reinterpret_cast<const float4 *>(binned->sorted4);
-    float *out[4] = {gx, gy, gz, gm};
-    for (int c = 0; c < (gm ? 4 : 3); ++c) {
-        k_adj_sym_finish<<<g, 256, 0, st>>>(mesh->N, F.acc + c * mesh->N, binned->perm, pos, binned->mass_varies,
-                                            c == 3, n_dense, out[c]);
-        HACC_LAUNCH_CHECK();
-    }
-    return HACC_OK;
+    float *const out[4] = {gx, gy, gz, gm};
+    return finish_totals(a, F.acc, n_dense, out, gm ? 4 : 3, binned->mass_varies, st);
 }
