@@ -27,9 +27,9 @@
 // A batch whose fullest lane holds more hits than HITS_DENSE of its records (a
 // halo next door) is evaluated densely from the same tile instead.  Measured
 // (GB300), gather force and adjoint with dL/dm: 2.1M lattice particles 1.83 ->
-// 0.90 ms and 3.17 -> 1.42 ms, 4096 uniform ones 85 -> 68 us; 16.8M clustered
+// 0.92 ms and 3.17 -> 1.45 ms, 4096 uniform ones 85 -> 69 us; 16.8M clustered
 // 63.2 -> 59.1 ms for the force, whose small cells alone take this path.
-// Symmetric force and adjoint, lattice: 1.24 -> 0.91 ms and 2.20 -> 1.35 ms.
+// Symmetric force and adjoint, lattice: 1.24 -> 0.96 ms and 2.20 -> 1.38 ms.
 #pragma once
 
 #include "hacc_terms.cuh"
@@ -53,6 +53,7 @@ constexpr int HITS_CELL = 40;
 // cotangents (adjoint), their n_j, and the mask words, each with the address
 // of its column.
 constexpr int HITS_PAD = 128;
+constexpr float HITS_FAR = 1.0e18f;  // an empty record's coordinates: outside any cutoff, squares finite
 __host__ __device__ constexpr int hits_lam_off() { return HITS_PAD + HITS_RECS * 16; }
 __host__ __device__ constexpr int hits_n_off(int mode)
 {
@@ -138,8 +139,10 @@ __device__ __forceinline__ void local_cell(uint32_t lc, uint32_t n, int &cx, int
     cz = (int)z;
 }
 
-// One i's sums: float32 over at most HITS_FOLD pairs, then compensated.
-constexpr int HITS_FOLD = 64;
+// One i's sums: float32 over at most HITS_FOLD pairs, then compensated.  Folds
+// of 64 left 2.2e-7 rms against float64 on the lattice, of 16 1.8e-7 (the dense
+// symmetric kernel 1.9e-7), for 2 % of the time.
+constexpr int HITS_FOLD = 16;
 
 template <int MODE>
 struct HitAcc {
@@ -204,7 +207,7 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
         bulk_copy(rows, a.pos + ib, (uint32_t)(ie - ib) * 16u, bar);
     }
     // records outside any cutoff ahead of the tile, and the end of the word list
-    if (lane < HITS_PAD / 16) sts128(base + 16 * lane, make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.f));
+    if (lane < HITS_PAD / 16) sts128(base + 16 * lane, make_float4(HITS_FAR, HITS_FAR, HITS_FAR, 0.f));
     for (int k = 0; k < HITS_STOPS; ++k) sts64(words + (NW + k) * 256, 0u, tile);
     const int row = g + 8 * (half ? q & 1 : q);
     i_own = ib + row;
@@ -281,8 +284,8 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
             // ---- 1. stage the batch in the i cell's frame, U entries' loads in flight together
             __syncwarp();  // the previous batch has been read
             if (lane < nb8 - nb) {  // fill the last step with records outside any cutoff
-                sts128(tile + 16 * (nb + lane), make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.f));
-                sts32(base + hits_n_off(MODE) + 4 * (nb + lane), 1.0e30f);
+                sts128(tile + 16 * (nb + lane), make_float4(HITS_FAR, HITS_FAR, HITS_FAR, 0.f));
+                sts32(base + hits_n_off(MODE) + 4 * (nb + lane), 1.0e37f);
                 if constexpr (is_adjoint(MODE))
                     sts128(tile + HITS_RECS * 16 + 16 * (nb + lane), make_float4(0.f, 0.f, 0.f, 0.f));
             }
