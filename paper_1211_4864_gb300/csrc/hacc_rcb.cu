@@ -519,6 +519,12 @@ __device__ __forceinline__ long long gap2_steps(const int32_t *qi, const int32_t
 }
 
 // One thread per leaf: count (FILL = false) or write (FILL = true) its list.
+// A walk is a chain of dependent loads, and the lanes of a warp diverge: up to
+// this many leaves, which leave the GPU idle otherwise, four share a warp, more
+// fill it.  Lists of 176, 5,892 and 46,798 leaves: 0.74, 1.31, 1.90 ms with full
+// warps, 0.45, 0.98, 3.20 ms with four a warp.
+constexpr int WALK_FEW = 8192;
+
 template <bool FILL>
 __global__ void __launch_bounds__(128)
 k_rcb_walk(const hacc_volume *__restrict__ vols, int V, const int32_t *__restrict__ n_leaves,
@@ -532,12 +538,16 @@ k_rcb_walk(const hacc_volume *__restrict__ vols, int V, const int32_t *__restric
     const int nl = *n_leaves;
     const int nn = *n_nodes;
     unsigned long long mine = 0;
-    for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < leaf_cap;
-         l += (int64_t)gridDim.x * blockDim.x) {
-        if (l >= nl) {
-            if (!FILL) counts[l] = 0;
-            continue;
-        }
+    if (!FILL) {
+        for (int64_t l = nl + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < leaf_cap;
+             l += (int64_t)gridDim.x * blockDim.x)
+            counts[l] = 0;
+    }
+    // leaves per warp: see WALK_FEW
+    const int per = nl <= WALK_FEW ? 4 : 32, lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t l = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per + lane; lane < per && l < nl;
+         l += warps * per) {
         const int v = find_volume_by_particle(vols, V, leaf_start[l]);
         const hacc_volume &vol = vols[v];
         const double Ld = (double)vol.L;
