@@ -272,6 +272,9 @@ __device__ __forceinline__ bool run_task(const KArgs &a, Ring<MODE, JT, STAGES> 
             if constexpr (is_adjoint(MODE)) {
                 if (EQ || k > 2) return A.total(u, k);
                 return A.total(u, k) - self_term(K, oi[u].w, k == 0 ? li[u].x : k == 1 ? li[u].y : li[u].z);
+            } else if constexpr (MODE == POTENTIAL) {
+                // the sum met particle i itself once (d = 0, se = eps exactly): take that term out
+                return A.h[u][0] + A.l[u][0] - oi[u].w * pair_potential_of(K.eps, K);
             } else
                 return A.h[u][k] + A.l[u][k];
         };

@@ -11,9 +11,12 @@
 //      n_i + n_j - 2 x_i.x_j - (cut squared), whose sign bits are shifted into
 //      one 32-bit mask per (i, column of the 8);
 //   3. the masks are transposed so that every lane owns one i (with at most 16
-//      i, two lanes share one), and each lane walks its own set bits: one
-//      16-byte shared load and one pair term per bit, in the arithmetic and
-//      with the cutoff test of the dense loops.
+//      i, two lanes share one), the i's own record is taken out, and each lane
+//      walks its own set bits: one 16-byte shared load and one pair term per
+//      bit, in the arithmetic and with the cutoff test of the dense loops.  (A
+//      pair of a particle with itself would add 0 f(0) and 0 f'(0): NaN once the
+//      softening is so small that these overflow, and a rounded zero times
+//      f(0) in the adjoint when the masses differ.)
 // The filter never loses a pair: tf32 rounds x to 2^-11 and n_j to 2^-11, so
 // the product sum is off by at most (2^-10 + 2^-11 + 2^-17)(|x_i|^2 + |x_j|^2)
 // (2 |x_i||x_j| <= |x_i|^2 + |x_j|^2; the last term covers the float32
@@ -51,7 +54,7 @@ constexpr int HITS_CELL = 40;
 // Shared memory of the path (bytes from its base): a pad of records outside
 // any cutoff (read by lanes that have run out of bits), the records, their
 // cotangents (adjoint), their n_j, and the mask words, each with the address
-// of its column.
+// of its column, and one word that says which records are the i cell's own.
 constexpr int HITS_PAD = 128;
 constexpr float HITS_FAR = 1.0e18f;  // an empty record's coordinates: outside any cutoff, squares finite
 __host__ __device__ constexpr int hits_lam_off() { return HITS_PAD + HITS_RECS * 16; }
@@ -62,7 +65,8 @@ __host__ __device__ constexpr int hits_n_off(int mode)
 __host__ __device__ constexpr int hits_word_off(int mode) { return hits_n_off(mode) + HITS_RECS * 4; }
 // ... eight words a lane and HITS_STOPS empty ones behind them
 constexpr int HITS_STOPS = 4;
-__host__ __device__ constexpr int hits_bytes(int mode) { return hits_word_off(mode) + (8 + HITS_STOPS) * 256; }
+__host__ __device__ constexpr int hits_own_off(int mode) { return hits_word_off(mode) + (8 + HITS_STOPS) * 256; }
+__host__ __device__ constexpr int hits_bytes(int mode) { return hits_own_off(mode) + 16; }
 
 __device__ __forceinline__ float4 lds128(uint32_t a)
 {
@@ -87,6 +91,16 @@ __device__ __forceinline__ void sts128(uint32_t a, float4 v)
 __device__ __forceinline__ void sts32(uint32_t a, float v)
 {
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t lds32u(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32u(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y)
 {
@@ -245,19 +259,22 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
     const float mi = unit ? 1.0f : oi.w;
     const uint32_t ones = q < 2 ? __float_as_uint(1.0f) : 0u;
 
-    const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
+    const int64_t e0 = a.nbr_off[c];
+    const int ne = (int)(a.nbr_off[c + 1] - e0);
 #pragma unroll 1
-    for (int64_t g0 = e0; g0 < e1; g0 += 32) {
+    for (int g0 = 0; g0 < ne; g0 += 32) {
         // lane l describes one entry: its j range, image offset and place among the group's records.
         // The 27-cell stencil is taken in steps of ten entries, so that every nine of them hold each
         // x, each y and each z offset three times: a batch then holds about as many partners of every i.
-        const int ng = (int)min((int64_t)32, e1 - g0);
+        const int ng = min(32, ne - g0);
         int jb = 0, cnt = 0;
         float Dx = 0.f, Dy = 0.f, Dz = 0.f;
+        bool home = false;  // the i cell itself
         if (lane < ng) {
-            const int64_t e = g0 + (ng == 27 ? lane * 10 % 27 : lane);
+            const int64_t e = e0 + g0 + (ng == 27 ? lane * 10 % 27 : lane);
             const int cp = a.nbr_cell[e];
             const int sh = a.nbr_shift[e];
+            home = cp == c && sh == 13;
             jb = a.cell_start[cp];
             cnt = a.cell_start[cp + 1] - jb;
             if (small_only && cnt > HITS_CELL) cnt = 0;
@@ -275,6 +292,10 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
         }
         const int total = __shfl_sync(FULL, first, 31);
         first -= cnt;
+        // the particle that record 0 would be in the i cell's own entry (none: out of every lane's reach)
+        if (lane == 0) sts32u(base + hits_own_off(MODE), 0x7fffffff);
+        __syncwarp();
+        if (home) sts32u(base + hits_own_off(MODE), (uint32_t)(jb - first));
 
 #pragma unroll 1
         for (int t0 = 0; t0 < total; t0 += HITS_RECS) {
@@ -298,7 +319,8 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
                     if constexpr (is_adjoint(MODE)) sts128(tile + HITS_RECS * 16 + 16 * r, l);
                 }
             };
-            constexpr int U = is_adjoint(MODE) ? 2 : 3;
+            // (2.1M lattice particles: force 925 us with two, 944 with three; potential 853 and 845)
+            constexpr int U = MODE == POTENTIAL ? 3 : 2;
             const int place = (at - t0) | n_own << 16;
             unsigned act = __ballot_sync(FULL, n_own > 0);
 #pragma unroll 1
@@ -386,10 +408,22 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
                     sts64(words + 256 * ((2 * s + k) ^ (g & 1)), v, tile + 16 * (2 * (q ^ s) + k));
                 }
             }
+            // no pair of an i with itself: its own record, if it is in this batch, loses its bit (such a
+            // batch never runs densely)
+            const uint32_t own = (uint32_t)(i_own - t0) - lds32u(base + hits_own_off(MODE));
+            if (own < (uint32_t)nb) {
+                const uint32_t s = ((own >> 1) & 3) ^ q;  // the lane's slot of column own mod 8 (half: 2, 3 are the other lane's)
+                if (s < (half ? 2u : 4u)) {
+                    const uint32_t w = words + 256 * ((2 * s + (own & 1)) ^ (g & 1));
+                    const uint32_t v = lds32u(w), v2 = v & ~(1u << (own >> 3));
+                    sts32u(w, v2);
+                    trips -= max(__popc(v), 1) - max(__popc(v2), 1);
+                }
+            }
             trips = __reduce_max_sync(FULL, trips);
             __syncwarp();
             // ---- 3. the pairs
-            if ((float)trips < HITS_DENSE * (float)(half ? nb8 / 2 : nb8)) {
+            if ((float)trips < HITS_DENSE * (float)(half ? nb8 / 2 : nb8) || __any_sync(FULL, own < (uint32_t)nb)) {
                 uint32_t mask, col, wp = words + 256;
                 asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mask), "=r"(col) : "r"(words) : "memory");
                 const uint32_t wend = words + NW * 256;
@@ -439,13 +473,6 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
             A.l[k] = __fadd_rn(A.l[k], l2);
         }
         active = active && q < 2;
-    }
-    if constexpr (is_adjoint(MODE)) {
-        if (!unit) {
-            A.l[0] -= self_term(K, oi.w, li.x);
-            A.l[1] -= self_term(K, oi.w, li.y);
-            A.l[2] -= self_term(K, oi.w, li.z);
-        }
     }
     __syncwarp();
     fence_async_proxy();  // the region's next use may be a bulk copy

@@ -124,7 +124,7 @@ __device__ __forceinline__ void pair_adjoint(const float4 p, const float4 l, flo
     }
 }
 
-// What a gather adjoint's sum W holds of the pair of i with itself (d = 0)
+// What a dense gather adjoint's sum W holds of the pair of i with itself (d = 0)
 // when the masses differ: f(0) times the rounding of m_i lam_i - m_i lam_i,
 // some 1e-4 for the default softening, taken out of the total again.
 __device__ __forceinline__ float self_term(const PairConsts &K, float m, float l)
@@ -140,8 +140,7 @@ template <int MODE, class Total>
 __device__ __forceinline__ void store_out(const KArgs &a, int o, const float4 &oi, bool eq, const Total &total)
 {
     if constexpr (MODE == POTENTIAL) {
-        // the sum met particle i itself once (d = 0, se = eps exactly): take that term out
-        a.out_x[o] = total(0) - oi.w * pair_potential_of(a.k.eps, a.k);
+        a.out_x[o] = total(0);
     } else {
         // equal masses: the sums times m
         const float sc = eq ? oi.w : 1.0f;
