@@ -296,7 +296,7 @@ __host__ __device__ constexpr int min_ctas(int mode) { return is_adjoint(mode) ?
 template <int MODE, int JT, int STAGES, bool EQ>
 __device__ __forceinline__ void dense_tasks(const KArgs &a, Ring<MODE, JT, STAGES> &ring, float *comp, int lane)
 {
-    const int ntask = *a.n_items;
+    const int ntask = dense_items(a);
     while (true) {
         int t = 0;
         if (lane == 0) t = atomicAdd(a.counter, 1);

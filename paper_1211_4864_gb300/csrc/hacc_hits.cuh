@@ -496,9 +496,6 @@ __device__ __forceinline__ bool hits_cell(const KArgs &a, int c, bool one_sided)
     const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
     int64_t nj = 0;
     for (int64_t e = e0; e < e1; ++e) {
-#ifdef HACC_DEBUG_BOUNDS
-        if (a.nbr_cell[e] < 0 || a.nbr_cell[e] >= a.n_cells) continue;  // reported when the task is taken
-#endif
         nj += a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
     }
     return nj <= 27 * HITS_CELL;
@@ -566,9 +563,6 @@ __device__ __forceinline__ int dense_reach(const KArgs &a, const int4 &task)
     int64_t nj = a.cell_start[task.x + 1] - task.z;
     for (int64_t e = first_entry(a, e0, mid); e < e1; ++e) {
         if (e == mid) continue;
-#ifdef HACC_DEBUG_BOUNDS
-        if (!a.origin && (a.nbr_cell[e] < 0 || a.nbr_cell[e] >= a.n_cells)) continue;  // reported when taken
-#endif
         const int cnt = a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
         if (takes_entry(e, mid, cnt)) nj += cnt;
     }
@@ -589,18 +583,15 @@ k_split_tasks(const KArgs a, bool one_sided, int2 *__restrict__ items, int32_t *
         const int oi = t < nt ? a.order[t] : -1;
         int kind = 0, n = 0, scale = 0;  // items of the thread's task, for the dense (0) or the hit kernel (1)
         if (t < nt) {
-            bool ok = true;
 #ifdef HACC_DEBUG_BOUNDS
-            ok = oi >= 0 && oi < a.task_cap;
-            if (ok) {
-                const int4 task = a.tasks[oi];
-                ok = task.w >= 0 && task.w < a.V && task.y < task.z && task.x >= 0 &&
-                     (a.origin || task.x < a.n_cells);
-            }
-            if (!ok) atomicOr(a.status, HACC_STATUS_BOUNDS);
+            int4 task;
+            const bool ok = task_in_bounds(a, oi, 0, 1, task);
+            if (!ok) report_bounds(a);
+#else
+            constexpr bool ok = true;
+            const int4 task = a.tasks[oi];
 #endif
             if (ok) {
-                const int4 task = a.tasks[oi];
                 kind = !a.origin && hits_cell(a, task.x, one_sided) ? 1 : 0;
                 n = kind || one_sided ? 1 : segment_count(a, task.z - task.y, dense_reach(a, task), scale);
             }
@@ -632,6 +623,9 @@ k_split_tasks(const KArgs a, bool one_sided, int2 *__restrict__ items, int32_t *
         }
         __syncthreads();
         const int64_t slot = (int64_t)base[kind] + wsum[kind][warp] + before[kind];
+#ifdef HACC_DEBUG_BOUNDS
+        if (slot + n > a.N) report_bounds(a);
+#endif
         for (int s = 0; s < n; ++s)
             if (slot + s < a.N) items[kind ? a.N - 1 - slot : slot + s] = make_int2(oi, s | scale << 16 | (s == n - 1 ? 1 << 24 : 0));
         __syncthreads();  // wsum and base are reused
@@ -688,7 +682,7 @@ __device__ __forceinline__ HitWarp hits_warp(unsigned char *smem, int warp, int 
 template <class Run>
 __device__ __forceinline__ void hits_tasks(const KArgs &a, int lane, const Run &run)
 {
-    const int nt = a.hit_count[2];
+    const int nt = hit_tasks(a);
     while (true) {
         int t = 0;
         if (lane == 0) t = atomicAdd(a.hit_count, 1);

@@ -127,58 +127,83 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long lo
 // neighbour list with the slot range that entry names -- and skips a task
 // that fails with HACC_STATUS_BOUNDS set, so that corrupted lists or tasks
 // never turn into out-of-range accesses.  (Tree lists are checked up to the
-// volume: the leaf count lives on the device.)  Warp-uniform.
+// task's slots: the leaf count lives on the device.)  The split (hacc_hits.cuh) and
+// every kernel that takes tasks make the check before they use one.
+#ifdef HACC_DEBUG_BOUNDS
+__device__ __forceinline__ void report_bounds(const KArgs &a)
+{
+    if (a.status) atomicOr(a.status, HACC_STATUS_BOUNDS);
+}
+
+// Task oi in bounds: this thread's share of the check, list entries first, first + step, ...
+__device__ __forceinline__ bool task_in_bounds(const KArgs &a, int oi, int first, int step, int4 &task)
+{
+    bool ok = oi >= 0 && oi < a.task_cap;
+    task = ok ? a.tasks[oi] : make_int4(0, 0, 0, 0);
+    ok = ok && task.w >= 0 && task.w < a.V && 0 <= task.y && task.y < task.z && task.z <= a.N;
+    if (!ok || a.origin) return ok;
+    const hacc_volume &vol = a.vols[task.w];
+    const int64_t cb = vol.cell_base, ce = vol.cell_base + (int64_t)vol.n * vol.n * vol.n;
+    if (!(task.x >= cb && task.x < ce && ce <= a.n_cells)) return false;
+    const int s0 = a.cell_start[task.x], s1 = a.cell_start[task.x + 1];
+    if (!(0 <= s0 && s0 <= task.y && task.z <= s1 && s1 <= a.N)) return false;
+    const int64_t e0 = a.nbr_off[task.x], e1 = a.nbr_off[task.x + 1];
+    if (!(e0 >= 0 && e1 == e0 + vol.S && e1 <= a.n_entries)) return false;
+    for (int64_t e = e0 + first; e < e1; e += step) {
+        const int cp = a.nbr_cell[e];
+        const int sh = a.nbr_shift[e];
+        if (!(cp >= cb && cp < ce && sh >= 0 && sh < 27)) return false;
+        const int j0 = a.cell_start[cp], j1 = a.cell_start[cp + 1];
+        if (!(0 <= j0 && j0 <= j1 && j1 <= a.N)) return false;
+    }
+    return true;
+}
+#endif
+
 __device__ __forceinline__ int task_count(const KArgs &a)
 {
     const int nt = *a.n_tasks;
 #ifdef HACC_DEBUG_BOUNDS
     if (nt < 0 || nt > a.task_cap) {
-        if ((threadIdx.x & 31) == 0) atomicOr(a.status, HACC_STATUS_BOUNDS);
+        if ((threadIdx.x & 31) == 0) report_bounds(a);
         return nt < 0 ? 0 : (int)a.task_cap;
     }
 #endif
     return nt;
 }
 
+// Warp-uniform.
 __device__ __forceinline__ bool take_task(const KArgs &a, int oi, int lane, int4 &task)
 {
 #ifndef HACC_DEBUG_BOUNDS
     task = a.tasks[oi];
     return true;
 #else
-    bool ok = oi >= 0 && oi < a.task_cap;
-    task = ok ? a.tasks[oi] : make_int4(0, 0, 0, 0);
-    ok = ok && task.w >= 0 && task.w < a.V;
-    if (ok && !a.origin) {
-        const hacc_volume &vol = a.vols[task.w];
-        const int64_t cb = vol.cell_base, ce = vol.cell_base + (int64_t)vol.n * vol.n * vol.n;
-        ok = task.x >= cb && task.x < ce && ce <= a.n_cells;
-        if (ok) {
-            const int s0 = a.cell_start[task.x], s1 = a.cell_start[task.x + 1];
-            ok = 0 <= s0 && s0 <= task.y && task.y < task.z && task.z <= s1 && s1 <= a.N;
-        }
-        if (ok) {
-            const int64_t e0 = a.nbr_off[task.x], e1 = a.nbr_off[task.x + 1];
-            ok = e0 >= 0 && e1 == e0 + vol.S && e1 <= a.n_entries;
-            if (ok) {
-                bool lane_ok = true;
-                for (int64_t e = e0 + lane; e < e1; e += 32) {
-                    const int cp = a.nbr_cell[e];
-                    const int sh = a.nbr_shift[e];
-                    bool eok = cp >= cb && cp < ce && sh >= 0 && sh < 27;
-                    if (eok) {
-                        const int j0 = a.cell_start[cp], j1 = a.cell_start[cp + 1];
-                        eok = 0 <= j0 && j0 <= j1 && j1 <= a.N;
-                    }
-                    lane_ok = lane_ok && eok;
-                }
-                ok = __all_sync(FULL, lane_ok);
-            }
-        }
-    }
-    ok = __all_sync(FULL, ok);
-    if (!ok && lane == 0) atomicOr(a.status, HACC_STATUS_BOUNDS);
+    const bool ok = __all_sync(FULL, task_in_bounds(a, oi, lane, 32, task));
+    if (!ok && lane == 0) report_bounds(a);
     return ok;
+#endif
+}
+
+// The split's results: the dense kernel's items and the hit kernel's tasks,
+// one slot each from the two ends of N slots.  (Debug build: the slots in use.
+// They run out when an order entry repeats; the split reports that.)
+__device__ __forceinline__ int dense_items(const KArgs &a)
+{
+#ifdef HACC_DEBUG_BOUNDS
+    return (int)min((int64_t)*a.n_items, a.N);
+#else
+    return *a.n_items;
+#endif
+}
+__device__ __forceinline__ int hit_tasks(const KArgs &a)
+{
+#ifdef HACC_DEBUG_BOUNDS
+    const int n = a.hit_count[2], room = (int)a.N - dense_items(a);
+    if (n > room && (threadIdx.x & 31) == 0) report_bounds(a);
+    return min(n, room);
+#else
+    return a.hit_count[2];
 #endif
 }
 

@@ -403,7 +403,7 @@ template <int JT, int STAGES, bool EQ>
 __device__ __forceinline__ void sym_tasks(const KArgs &a, Ring<FORCE, JT, STAGES> &ring, float *comp, double *acc,
                                           int64_t N, int lane)
 {
-    const int ntask = *a.n_items;
+    const int ntask = dense_items(a);
     while (true) {
         int t = 0;
         if (lane == 0) t = atomicAdd(a.counter, 1);

@@ -285,7 +285,7 @@ template <int JT, int STAGES, bool GM, bool EQ>
 __device__ __forceinline__ void adj_sym_tasks(const KArgs &a, Ring<ADJOINT, JT, STAGES> &ring, float *comp,
                                               double *acc, int64_t N, int lane)
 {
-    const int ntask = *a.n_items;
+    const int ntask = dense_items(a);
     while (true) {
         int t = 0;
         if (lane == 0) t = atomicAdd(a.counter, 1);

@@ -9,7 +9,8 @@ bit); on lists or tasks corrupted on purpose it must report the corruption
 instead of reading out of range, and the next call on rebuilt lists must be
 clean again.  The corruptions stay inside the arrays: only the values that
 the kernels would use as indices are wrong, and the checks run before any such
-value is used.
+value is used, in the kernel that splits the tasks (it walks the lists first)
+and again in the pair kernels.
 """
 
 import numpy as np
@@ -120,7 +121,9 @@ def test_debug_build_binning_is_the_product_binning(torch, hs):
         assert np.array_equal(g.view(np.int32), r.view(np.int32))
 
 
-@pytest.mark.parametrize("what", ["list entry", "list image code", "task slots", "task count"])
+@pytest.mark.parametrize("what", ["list entry", "list image code", "task slots", "task count",
+                                  "list beyond the entries", "list before the entries", "list length",
+                                  "cell start beyond the particles", "task of no particles", "order entry"])
 def test_corrupted_lists_and_tasks_are_reported_not_read(torch, hs, debug_lib, what):
     w, c, prm, sr, pos, m, lam = _case(torch, hs, seed=22)
     sr.prepare(pos, m)
@@ -133,6 +136,19 @@ def test_corrupted_lists_and_tasks_are_reported_not_read(torch, hs, debug_lib, w
     elif what == "task slots":
         k = int(sr.task_order[3].item())
         sr.tasks[k, 2] = w.N + 50
+    elif what in ("list beyond the entries", "list before the entries"):
+        S = int((sr.nbr_off[1] - sr.nbr_off[0]).item())
+        sr.nbr_off[9] = sr.n_entries + (1 << 40) if "beyond" in what else -(1 << 40)
+        sr.nbr_off[10] = sr.nbr_off[9] + S
+    elif what == "list length":
+        sr.nbr_off[12] = sr.nbr_off[11] + (1 << 33)
+    elif what == "cell start beyond the particles":
+        sr.cell_start[20] = (1 << 31) - 5
+    elif what == "task of no particles":
+        k = int(sr.task_order[5].item())
+        sr.tasks[k, 2] = sr.tasks[k, 1]
+    elif what == "order entry":
+        sr.task_order[7] = sr.task_cap + (1 << 28)
     else:
         sr.n_tasks[0] = sr.task_cap + 5
     for name, call in (("force", lambda: sr.force(prm)), ("force_symmetric", lambda: sr.force_symmetric(prm)),
@@ -153,3 +169,28 @@ def test_corrupted_lists_and_tasks_are_reported_not_read(torch, hs, debug_lib, w
     A = oracle.sr_force(w.x, w.y, w.z, w.m, 16.0, EPS, RC, c.astype(np.float64))
     rms, _ = err_norms(a.cpu().numpy().T, A)
     assert rms < RMS_TOL
+
+
+@pytest.mark.parametrize("call", ["force_symmetric", "adjoint_symmetric"])
+def test_repeated_order_entries_do_not_overrun_the_items(torch, hs, debug_lib, call):
+    """One particle in each of 8,000 cells and 8,000 in one: a full task of that cell becomes some 31 segments, so order
+    entries that all name it ask for sixteen times the N item slots.  Only N are written and taken, and the call says
+    so."""
+    rng = np.random.default_rng(4)
+    g = np.stack(np.meshgrid(*[np.arange(20)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pos = np.concatenate([g + rng.uniform(0.1, 0.9, g.shape), g[4210] + rng.uniform(0.1, 0.9, (8000, 3))]) * 3.0
+    N = len(pos)
+    sr = hs.ShortRange(60.0, np.array([0, N]), RC, split_T=128)
+    sr.prepare(torch.tensor(pos.T.astype(np.float32).copy(), device="cuda"), torch.ones(N, device="cuda"))
+    torch.cuda.synchronize()
+    sr.check_status()
+    nt = int(sr.n_tasks.item())
+    size = sr.tasks[:nt, 2] - sr.tasks[:nt, 1]
+    sr.task_order[:nt] = int(torch.argmax(size).item())
+    prm = hs.SRParams(EPS, RC, default_coeffs(RC, EPS))
+    if call == "force_symmetric":
+        sr.force_symmetric(prm)
+    else:
+        sr.adjoint_symmetric(prm, torch.ones(3, N, device="cuda"))
+    torch.cuda.synchronize()
+    assert hs.hacc_get_status(sr.status) & BOUNDS
