@@ -508,7 +508,8 @@ extern "C" int hacc_sr_force_symmetric(const hacc_mesh *mesh, const hacc_binned 
     rc = split_tasks(a, F, false, st);
     if (rc) return rc;
     const int32_t *n_dense = a.n_items;
-    rc = zero_totals(a, F.acc, 3, n_dense, st);
+    float *const out[4] = {ax, ay, az, nullptr};
+    rc = zero_totals(a, F.acc, out, 3, n_dense, st);
     if (rc) return rc;
     hacc_launch L;
     if (launch) {
@@ -527,6 +528,5 @@ extern "C" int hacc_sr_force_symmetric(const hacc_mesh *mesh, const hacc_binned 
         rc = launch_hits(k_hits_sym<FORCE>, FORCE, st, a, F.acc);
         if (rc) return rc;
     }
-    float *const out[4] = {ax, ay, az, nullptr};
     return finish_totals(a, F.acc, n_dense, out, 3, nullptr, st);
 }

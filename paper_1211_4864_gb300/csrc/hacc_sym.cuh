@@ -64,24 +64,36 @@ __device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, i
 }
 
 // Without dense tasks (n_dense given and 0) the hit kernel stores every
-// output itself: the totals are then neither zeroed nor converted.
+// task's outputs itself: the totals are then neither zeroed nor converted.
 __device__ __forceinline__ bool no_totals(const int32_t *n_dense) { return n_dense && *n_dense == 0; }
 
+struct TotalsOut {
+    float *out[4];
+};
+
+// Zeroes the totals or, when the hit kernel stores, the outputs: a particle
+// whose task was dropped (a task buffer too small, a wait that ran out) reads
+// 0 on both ways.
 __global__ void __launch_bounds__(256)
-k_zero_totals(double2 *__restrict__ acc, int64_t n2, const int32_t *__restrict__ n_dense)
+k_zero_totals(double2 *__restrict__ acc, int64_t n2, const int32_t *__restrict__ n_dense, TotalsOut o, int nc, int64_t N)
 {
-    if (no_totals(n_dense)) return;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n2; k += (int64_t)gridDim.x * blockDim.x)
-        acc[k] = make_double2(0.0, 0.0);
+    const int64_t k0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (no_totals(n_dense)) {
+        for (int c = 0; c < nc; ++c)
+            for (int64_t k = k0; k < N; k += step) o.out[c][k] = 0.0f;
+        return;
+    }
+    for (int64_t k = k0; k < n2; k += step) acc[k] = make_double2(0.0, 0.0);
 }
 
 // Zeroes nc totals per particle (the region holds SYM_ACC_MAX of them).
-int zero_totals(const KArgs &a, double *acc, int nc, const int32_t *n_dense, cudaStream_t st)
+int zero_totals(const KArgs &a, double *acc, float *const (&out)[4], int nc, const int32_t *n_dense, cudaStream_t st)
 {
     const int64_t n2 = (a.N * nc + 1) / 2;
     int64_t g = (n2 + 255) / 256;
     if (g > num_sms() * 16) g = num_sms() * 16;
-    k_zero_totals<<<(int)g, 256, 0, st>>>(reinterpret_cast<double2 *>(acc), n2, n_dense);
+    const TotalsOut o{{out[0], out[1], out[2], out[3]}};
+    k_zero_totals<<<(int)g, 256, 0, st>>>(reinterpret_cast<double2 *>(acc), n2, n_dense, o, nc, a.N);
     HACC_LAUNCH_CHECK();
     return HACC_OK;
 }
@@ -95,9 +107,6 @@ int zero_totals(const KArgs &a, double *acc, int nc, const int32_t *n_dense, cud
 // not (each partial sector is then read and written back in DRAM: 0.82 against
 // 0.33 ms).  The streamed totals and perm are loaded evict-first for the same
 // reason.
-struct TotalsOut {
-    float *out[4];
-};
 __global__ void __launch_bounds__(256)
 k_finish_totals(int64_t N, const double *__restrict__ acc, const int32_t *__restrict__ perm,
                 const float4 *__restrict__ pos, const uint32_t *mass_varies,

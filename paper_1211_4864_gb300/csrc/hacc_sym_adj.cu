@@ -398,7 +398,8 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
     rc = split_tasks(a, F, false, st);
     if (rc) return rc;
     const int32_t *n_dense = a.n_items;
-    rc = zero_totals(a, F.acc, gm ? 4 : 3, n_dense, st);
+    float *const out[4] = {gx, gy, gz, gm};
+    rc = zero_totals(a, F.acc, out, gm ? 4 : 3, n_dense, st);
     if (rc) return rc;
     hacc_launch L;
     if (launch) {
@@ -418,6 +419,5 @@ extern "C" int hacc_sr_force_adjoint_symmetric(const hacc_mesh *mesh, const hacc
                 : launch_hits(k_hits_sym<ADJOINT>, ADJOINT, st, a, F.acc);
         if (rc) return rc;
     }
-    float *const out[4] = {gx, gy, gz, gm};
     return finish_totals(a, F.acc, n_dense, out, gm ? 4 : 3, binned->mass_varies, st);
 }

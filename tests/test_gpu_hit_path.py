@@ -101,3 +101,31 @@ def test_cells_of_every_size(n, side, big, cell_min, split_T, masses):
     if n >= 8:
         assert np.linalg.norm(phi.cpu().numpy() - P) / np.linalg.norm(P) < RMS_TOL
     assert torch.equal(a, again)
+
+
+@pytest.mark.parametrize("what", ["tasks dropped", "wait runs out"])
+def test_outputs_of_tasks_that_did_not_run_are_zero(what):
+    """Small cells only: every output of a symmetric call is written, 0 where a task was dropped (and flagged)."""
+    torch = need_cuda()
+    import paper_1211_4864_gb300 as hs
+    hs.load()
+    pos, L = cells(9, 5, seed=2)
+    N = len(pos)
+    sr = hs.ShortRange(L, np.array([0, N]), RC)
+    prm = hs.SRParams(EPS, RC, default_coeffs(RC, EPS))
+    lam = torch.ones(3, N, device="cuda")
+    if what == "tasks dropped":
+        sr.lists.task_cap = 5
+    sr.prepare(torch.tensor(pos.T.copy(), device="cuda"), torch.ones(N, device="cuda"))
+    torch.cuda.synchronize()
+    sr.status.zero_()
+    launch = hs.Launch(wait_cycles=1) if what == "wait runs out" else None
+    outs = [torch.full((3, N), float("nan"), device="cuda") for _ in range(2)]
+    sr.force_symmetric(prm, outs[0], launch=launch)
+    sr.adjoint_symmetric(prm, lam, outs[1], launch=launch)
+    torch.cuda.synchronize()
+    done = 45 if what == "tasks dropped" else 0  # five tasks of one cell's nine particles
+    for out in outs:
+        o = out.cpu().numpy()
+        assert np.all(np.isfinite(o))
+        assert np.count_nonzero(np.any(o != 0, axis=0)) <= done
