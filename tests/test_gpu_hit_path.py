@@ -129,3 +129,34 @@ def test_outputs_of_tasks_that_did_not_run_are_zero(what):
         o = out.cpu().numpy()
         assert np.all(np.isfinite(o))
         assert np.count_nonzero(np.any(o != 0, axis=0)) <= done
+
+
+@pytest.mark.parametrize("masses", ["equal", "varied"])
+def test_stored_and_converted_totals_are_the_same_numbers(masses):
+    """A symmetric call's outputs for small cells do not depend on whether a dense cell elsewhere has the sums go through
+    the float64 totals: the hit kernel's own stores round the same products once.  (Its product of a mass and a
+    two-word sum is exact to 2^-46, so at most one value in 2^20 falls on the other side of a tie.)"""
+    torch = need_cuda()
+    import paper_1211_4864_gb300 as hs
+    hs.load()
+    small, L = cells(20, 8, seed=6)
+    rng = np.random.default_rng(8)
+    blob = (0.01 + 2.98 * rng.random((300, 3))).astype(np.float32)  # one cell, dense
+    own = np.all(small >= 6.0, axis=1) & np.all(small < 21.0, axis=1)  # no neighbour of that cell's
+    m = rng.uniform(0.5, 2.0, len(small) + 300).astype(np.float32) if masses == "varied" else np.full(len(small) + 300, 0.37, np.float32)
+    lam = rng.normal(size=(3, len(small) + 300)).astype(np.float32)
+    prm = hs.SRParams(EPS, RC, default_coeffs(RC, EPS))
+    outs = []
+    for pos in (small, np.concatenate([small, blob])):
+        N = len(pos)
+        sr = hs.ShortRange(L, np.array([0, N]), RC)
+        sr.prepare(torch.tensor(pos.T.copy(), device="cuda"), torch.tensor(m[:N], device="cuda"))
+        lt = torch.tensor(lam[:, :N].copy(), device="cuda")
+        f = sr.force_symmetric(prm)
+        g, gm = sr.adjoint_symmetric(prm, lt)
+        w, _ = sr.adjoint_symmetric(prm, lt, want_gm=False)
+        torch.cuda.synchronize()
+        sr.check_status()
+        outs.append([t.cpu().numpy()[..., : len(small)][..., own] for t in (f, g, gm, w)])
+    for a, b in zip(*outs):
+        assert np.count_nonzero(a != b) <= 1 and np.allclose(a, b, rtol=2.0 ** -23, atol=0)
