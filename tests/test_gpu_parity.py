@@ -522,3 +522,25 @@ def test_moments_double_float_against_float64(torch, hs):
     # the same sums with v or a left out, and the order-fixed result repeats bit for bit
     got2 = sr.moments(dev(m), None, dev(a), None).cpu().numpy()
     assert np.all(got2[[0, 1, 2, 6, 8]] == 0.0) and np.array_equal(got2[[3, 4, 5, 7]], got[[3, 4, 5, 7]])
+
+
+def test_moments_of_sums_that_cancel(torch, hs):
+    """At 16.8M particles whose second half repeats the first with the velocities reversed, sum m v is zero.  A thread
+    adds 16 terms in double-float and rounds each running sum of k terms to 2^-48 of it, 2^-49 k / sqrt(3) of a term
+    rms: 21 x 2^-49 over the 16 if the sums only grow, 2^10 of that over the 2^20 threads, 2.3e-18 of the sum of
+    magnitudes (half the terms take a thread's sum back towards zero: 1e-18 is typical).  Threads of a hundred terms
+    leave up to 1.4e-17."""
+    from paper_1211_4864_gb300 import _lib
+    N, h = 1 << 24, 1 << 23
+    ws = torch.empty(int(_lib.load().hacc_moments_workspace_size(N)), dtype=torch.uint8, device="cuda")
+    for seed in range(3):
+        rng = np.random.default_rng(seed)
+        m = rng.uniform(0.5, 1.0, h).astype(np.float32)
+        u = rng.uniform(0.5, 1.0, (3, h)).astype(np.float32)
+        p = rng.permutation(h)
+        M = torch.tensor(np.concatenate([m, m[p]]), device="cuda")
+        V = torch.tensor(np.concatenate([u, -u[:, p]], 1), device="cuda")
+        out = torch.empty(9, dtype=torch.float64, device="cuda")
+        hs.hacc_moments(N, M, V[0], V[1], V[2], None, None, None, out, ws)
+        size = 2 * (m.astype(np.float64) * u).sum(1)
+        assert np.all(np.abs(out.cpu().numpy()[:3]) < 2.3e-18 * size)
