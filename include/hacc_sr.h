@@ -394,7 +394,9 @@ int hacc_sr_potential(const hacc_mesh *mesh, const hacc_binned *binned, const ha
 /* Counts, into the device int64 *out, the ordered pairs (j != i) that the
  * pair kernels find inside the cutoff: s + eps < r_c^2 + eps evaluated in
  * float32 on the cell-relative offsets exactly as hacc_sr_force evaluates it
- * (the paper's "short-range condition", Sec. III).  With the candidate count
+ * (the paper's "short-range condition", Sec. III; the symmetric call's dense
+ * cells round the offsets in another order, so a pair within rounding of r_c
+ * may differ there).  With the candidate count
  * of hacc_build_lists it gives the lists' efficiency.  A reporting tool, not
  * a hot path (one i per lane, j straight from global memory). */
 int hacc_count_pairs(const hacc_mesh *mesh, const hacc_binned *binned, const hacc_lists *lists,

@@ -386,10 +386,12 @@ __global__ void __launch_bounds__(HITS_WARPS * 32, hits_ctas(MODE)) k_hits(const
     wait_previous_kernel();
 }
 
-// Ordered pairs (j != i) inside the cutoff, decided exactly as the pair
-// kernels decide it (same offsets, same float32 s + eps, same compare).  One
-// warp per task, one i per lane, j read straight from global memory: a
-// reporting tool, not a hot path.
+// Ordered pairs (j != i) inside the cutoff, decided exactly as the gather
+// force decides it: same offsets, same float32 s + eps, same compare, and the
+// image offset added to j for the cells of the hit path, taken from i for the
+// dense kernel's (so a pair on the cutoff itself can be counted from one side
+// alone).  One warp per task, one i per lane, j read straight from global
+// memory: a reporting tool, not a hot path.
 __global__ void __launch_bounds__(256)
 k_count_pairs(const KArgs a, unsigned long long *__restrict__ total)
 {
@@ -407,6 +409,7 @@ k_count_pairs(const KArgs a, unsigned long long *__restrict__ total)
         const int64_t lc = (int64_t)task.x - vol.cell_base;
         const int cx = (int)(lc % n), cy = (int)((lc / n) % n), cz = (int)(lc / ((int64_t)n * n));
         const float4 org_i = a.origin ? a.origin[task.x] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool hit = !a.origin && hits_cell(a, task.x, true);
         for (int i = task.y + lane; i - lane < task.z; i += 32) {
             const bool active = i < task.z;
             const float4 oi = active ? a.pos[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -426,11 +429,17 @@ k_count_pairs(const KArgs a, unsigned long long *__restrict__ total)
                     Dx = (float)((double)cell_centre(px, w) - (double)cell_centre(cx, w) + sx * Ld);
                     Dy = (float)((double)cell_centre(py, w) - (double)cell_centre(cy, w) + sy * Ld);
                     Dz = (float)((double)cell_centre(pz, w) - (double)cell_centre(cz, w) + sz * Ld);
+                    if (hit) {
+                        Dx = image_delta(cell_centre(px, w), cell_centre(cx, w), (float)sx * vol.L);
+                        Dy = image_delta(cell_centre(py, w), cell_centre(cy, w), (float)sy * vol.L);
+                        Dz = image_delta(cell_centre(pz, w), cell_centre(cz, w), (float)sz * vol.L);
+                    }
                 }
                 const float oxp = oi.x - Dx, oyp = oi.y - Dy, ozp = oi.z - Dz;
                 for (int j = a.cell_start[cp]; j < a.cell_start[cp + 1]; ++j) {
                     const float4 p = a.pos[j];
-                    const float dx = p.x - oxp, dy = p.y - oyp, dz = p.z - ozp;
+                    const float dx = hit ? (p.x + Dx) - oi.x : p.x - oxp, dy = hit ? (p.y + Dy) - oi.y : p.y - oyp,
+                                dz = hit ? (p.z + Dz) - oi.z : p.z - ozp;
                     const float se = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, a.k.eps)));
                     cnt += (active && j != i && se < a.k.rc2e) ? 1ull : 0ull;
                 }

@@ -470,11 +470,12 @@ class ShortRange:
             raise HaccError(f"device status {s:#x}")
 
     def pair_count(self) -> int:
-        """Candidate ordered pairs (j != i) the pair kernels evaluate."""
+        """Candidate ordered pairs (j != i) of the lists.  (The pair kernels evaluate the term of each of them in
+        larger cells, and in small cells only of those near or inside the cutoff.)"""
         return int(self.n_pairs.item())
 
     def pairs_within_cutoff(self, params: SRParams) -> int:
-        """Ordered pairs (j != i) inside the cutoff, decided as the pair kernels decide."""
+        """Ordered pairs (j != i) inside the cutoff, decided as force() decides."""
         out = torch.zeros(1, dtype=torch.int64, device=self.device)
         hacc_count_pairs(self.mesh, self.binned, self.lists, params, out)
         return int(out.item())
