@@ -35,21 +35,11 @@ __device__ __forceinline__ void entry_delta(const KArgs &a, const hacc_volume &v
     }
 }
 
-// Lane's entry of the group at g0 (first record jb, cnt of them) clipped to
-// the segment's j records of the task's flattened list, whose entries start at
-// e_first.  size: the task's particles.
-__device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, int size, int64_t e_first, int64_t mid,
-                                           int64_t g0, int &jb, int &cnt, int own)
+// Lane's entry of a group (first record jb, cnt of them) clipped to the
+// segment's j records of the task's flattened list.  before: the records of
+// the groups before, brought up to date.  size: the task's particles.
+__device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, int size, int &before, int &jb, int &cnt)
 {
-    int before = 0;  // records of the groups before (lists of more than 32 entries)
-    for (int64_t e = e_first + lane; e < g0; e += 32) {
-        int n = own;
-        if (e != mid) {
-            n = a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];
-            if (!takes_entry(e, mid, n)) n = 0;
-        }
-        before += n;
-    }
     int inc = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -57,7 +47,8 @@ __device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, i
         if (lane >= o) inc += t;
     }
     const int per = segment_records(a, size) << ((code >> 16) & 31), jlo = (code & 0xffff) * per;
-    const int first = (int)__reduce_add_sync(FULL, (unsigned)before) + inc - cnt;
+    const int first = before + inc - cnt;
+    before += __shfl_sync(FULL, inc, 31);
     const int lo = max(first, jlo), hi = code >> 24 ? first + cnt : min(first + cnt, jlo + per);
     jb += lo - first;
     cnt = max(hi - lo, 0);

@@ -191,6 +191,7 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
     const int64_t e0 = a.nbr_off[c], e1 = a.nbr_off[c + 1];
     const int64_t mid = self_entry(a, c, e0, e1, vol);
     const int ce = a.cell_start[c + 1];
+    int before = 0;  // records of the list's groups before (segments)
     for (int64_t g0 = first_entry(a, e0, mid); g0 < e1; g0 += 32) {
         const int ng = (int)min((int64_t)32, e1 - g0);
         int jb = 0, cnt = 0;
@@ -207,8 +208,7 @@ __device__ __forceinline__ bool run_task_adj_sym(const KArgs &a, Ring<ADJOINT, J
                 entry_delta(a, vol, cp, a.nbr_shift[g0 + lane], cx, cy, cz, org_i, Dx, Dy, Dz);
             }
         }
-        if (code != SEG_WHOLE)
-            clip_entry(a, lane, code, ie - ib, first_entry(a, e0, mid), mid, g0, jb, cnt, ce - ie);
+        if (code != SEG_WHOLE) clip_entry(a, lane, code, ie - ib, before, jb, cnt);
         int pk = 0, poff = 0;
         int ck = 0, coff = 0;
         for (int s = 0; s < STAGES; ++s)

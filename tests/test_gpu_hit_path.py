@@ -34,7 +34,7 @@ def rounding_bounds(pos, m, lam, L):
     """Per particle, what the rounding of its pairs' terms can add to a force and to a gradient component.  With t =
     (s + eps)^-1/2 from a root within two units in the last place, t^3 is off by 2^-21 of itself and a Horner sum of
     terms whose magnitudes add to at most 6 (value) or 8 (slope times s) by 6 2^-24 of them; the offsets, below 8 in
-    magnitude, add 2^-22 to a distance."""
+    magnitude, add 2^-22 to a distance.  The third bound is for dL/dm."""
     d = pos[None] - pos[:, None]
     d -= L * np.round(d / L)
     s = (d * d).sum(-1)
@@ -44,7 +44,7 @@ def rounding_bounds(pos, m, lam, L):
     slope = 2.0 ** -21 * (8 * t ** 3 + 16) + 2.0 ** -22 * 16 * (t ** 4 + 1)
     l = np.linalg.norm(lam, axis=1)
     mu = m[:, None] * l[None] + m[None] * l[:, None]
-    return (near * m[None] * f).sum(1), (near * mu * slope).sum(1)
+    return (near * m[None] * f).sum(1), (near * mu * slope).sum(1), (near * f * l[None]).sum(1)
 
 
 CASES = [(1, 3, 0, 3.0, 32), (8, 3, 0, 3.0, 32), (9, 3, 0, 3.0, 32), (10, 4, 0, 3.0, 64), (16, 3, 0, 3.0, 32),
@@ -83,10 +83,12 @@ def test_cells_of_every_size(n, side, big, cell_min, split_T, masses):
     G, GM = oracle.sr_force_adjoint(*pos.T.copy(), m, L, EPS, RC, c64, lam.astype(np.float64))
     P = oracle.sr_potential(*pos.T.copy(), m, L, EPS, RC, c64)
     if n < 8:  # few pairs, most of them where f = t^3 - poly nearly cancels: the terms' own rounding
-        bf, bg = rounding_bounds(pos.astype(np.float64), m, lam, L)
+        bf, bg, bm = rounding_bounds(pos.astype(np.float64), m, lam, L)
         for name, t in got.items():
             err = np.abs(t.cpu().numpy().T - (G if "adjoint" in name else A)).max(1)
             assert np.all(err <= (bg if "adjoint" in name else bf) + 1e-9), name
+        for name, t in (("adjoint gm", gm), ("adjoint symmetric gm", gms)):
+            assert np.all(np.abs(t.cpu().numpy() - GM) <= bm + 1e-9), name
     else:
         for name, t in got.items():
             rms, mx = err_norms(t.cpu().numpy().T.astype(np.float64), G if "adjoint" in name else A)
@@ -160,3 +162,63 @@ def test_stored_and_converted_totals_are_the_same_numbers(masses):
         outs.append([t.cpu().numpy()[..., : len(small)][..., own] for t in (f, g, gm, w)])
     for a, b in zip(*outs):
         assert np.count_nonzero(a != b) <= 1 and np.allclose(a, b, rtol=2.0 ** -23, atol=0)
+
+
+def fine_mesh():
+    """Cells of half the cutoff (lists of up to 125 entries, four groups of 32): ten particles in each of 10^3, 3,003 in
+    two that are each other's neighbours and 50 in another, so that dense tasks skip large cells and meet small ones
+    before their own, over several groups."""
+    rng = np.random.default_rng(12)
+    g = np.stack(np.meshgrid(*[np.arange(10)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    n = np.full(1000, 10)
+    n[[444, 556]] = 3003
+    n[455] = 50
+    return (np.repeat(g, n, axis=0) + rng.uniform(0.01, 0.99, (n.sum(), 3))) * 1.5, 15.0, 1.5
+
+
+def crowded_cell():
+    """33,283 particles in one cell: its last task holds 3, and one particle of the next cells meets more than 32,768 j
+    records, so that a segment is a multiple of the usual length."""
+    rng = np.random.default_rng(13)
+    pos = np.concatenate([rng.uniform(3.001, 5.999, (128 * 260 + 3, 3)), rng.uniform(0.0, 9.0, (300, 3))])
+    out = np.all((pos[-300:] > 3.0) & (pos[-300:] < 6.0), axis=1)
+    return np.delete(pos, len(pos) - 300 + np.nonzero(out)[0], axis=0), 9.0, 3.0
+
+
+@pytest.mark.parametrize("field", [fine_mesh, crowded_cell])
+@pytest.mark.parametrize("masses", ["equal", "varied"])
+def test_segments_of_long_lists_and_full_cells(field, masses):
+    torch = need_cuda()
+    import paper_1211_4864_gb300 as hs
+    hs.load()
+    pos, L, cell_min = field()
+    rng = np.random.default_rng(14)
+    pos = pos[rng.permutation(len(pos))].astype(np.float32)
+    N = len(pos)
+    m = rng.uniform(0.5, 2.0, N).astype(np.float32) if masses == "varied" else np.full(N, 0.37, np.float32)
+    lam = rng.normal(size=(N, 3)).astype(np.float32)
+    c = default_coeffs(RC, EPS)
+    prm = hs.SRParams(EPS, RC, c)
+    sr = hs.ShortRange(L, np.array([0, N]), RC, cell_min=cell_min, split_T=128)
+    sr.prepare(torch.tensor(pos.T.copy(), device="cuda"), torch.tensor(m, device="cuda"))
+    lt = torch.tensor(lam.T.copy(), device="cuda")
+    a = sr.force_symmetric(prm)
+    g, gm = sr.adjoint_symmetric(prm, lt)
+    torch.cuda.synchronize()
+    sr.check_status()
+    start, perm = sr.cell_start.cpu().numpy(), sr.perm.cpu().numpy()
+    count = np.diff(start)
+    if field is fine_mesh:
+        assert sr.n_entries == 1000 * 125 and count.max() > 3000
+    else:
+        assert count.max() > 32768 and count.max() % 128 == 3
+    full = np.argsort(count)[-2:]
+    tail = np.concatenate([perm[start[k + 1] - 3 : start[k + 1]] for k in full])  # the short last tasks
+    t = np.unique(np.concatenate([rng.choice(N, 600, replace=False), tail, perm[start[full[1]] :][:128]]))
+    c64 = c.astype(np.float64)
+    A = oracle.sr_force(*pos.T.copy(), m, L, EPS, RC, c64, targets=t)
+    G, GM = oracle.sr_force_adjoint(*pos.T.copy(), m, L, EPS, RC, c64, lam.astype(np.float64), targets=t)
+    for name, got, ref in (("force", a, A), ("adjoint", g, G)):
+        rms, mx = err_norms(got.cpu().numpy().T[t].astype(np.float64), ref)
+        assert rms < RMS_TOL and mx < MAX_TOL, (name, rms, mx)
+    assert np.linalg.norm(gm.cpu().numpy()[t] - GM) < RMS_TOL * np.linalg.norm(GM)
