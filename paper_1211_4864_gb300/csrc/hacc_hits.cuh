@@ -555,12 +555,26 @@ __device__ __forceinline__ int64_t self_entry(const KArgs &a, int c, int64_t e0,
 __device__ __forceinline__ int64_t first_entry(const KArgs &a, int64_t e0, int64_t mid) { return a.origin ? mid : e0; }
 __device__ __forceinline__ bool takes_entry(int64_t e, int64_t mid, int cnt) { return e > mid || cnt <= HITS_CELL; }
 
-// The j records a symmetric call's dense task meets beyond its own chunk.
+// The j records a symmetric call's dense task meets beyond its own chunk.  A
+// tree's lists are long and its leaves alike (between half of the largest size
+// and all of it), so there sixteen entries stand for all: the last segment
+// takes whatever is left.  (Walked by one thread a task, the lists of 45,593
+// leaves of at most 8 took 665 us of the call's 5,640; of 5,892 leaves of at
+// most 64, 1.02 ms a call with exact counts, 0.95 with these.)
 __device__ __forceinline__ int dense_reach(const KArgs &a, const int4 &task)
 {
     const int64_t e0 = a.nbr_off[task.x], e1 = a.nbr_off[task.x + 1];
     const int64_t mid = self_entry(a, task.x, e0, e1, a.vols[task.w]);
     int64_t nj = a.cell_start[task.x + 1] - task.z;
+    if (a.origin && e1 - mid > 32) {
+        int some = 0;
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            const int cp = a.nbr_cell[mid + 1 + (e1 - mid - 1) * k / 16];
+            some += a.cell_start[cp + 1] - a.cell_start[cp];
+        }
+        return (int)min(nj + (e1 - mid - 1) * some / 16, (int64_t)1 << 30);
+    }
     for (int64_t e = first_entry(a, e0, mid); e < e1; ++e) {
         if (e == mid) continue;
         const int cnt = a.cell_start[a.nbr_cell[e] + 1] - a.cell_start[a.nbr_cell[e]];

@@ -310,10 +310,14 @@ __device__ __forceinline__ bool run_task_sym(const KArgs &a, Ring<FORCE, JT, STA
                 jb = a.cell_start[cp];
                 cnt = a.cell_start[cp + 1] - jb;
                 if (!takes_entry(g0 + lane, mid, cnt)) cnt = 0;
-                entry_delta(a, vol, cp, a.nbr_shift[g0 + lane], cx, cy, cz, org_i, Dx, Dy, Dz);
             }
         }
-        if (code != SEG_WHOLE) clip_entry(a, lane, code, ie - ib, before, jb, cnt);
+        if (code != SEG_WHOLE) {
+            if (!clip_entry(a, lane, code, ie - ib, before, jb, cnt)) break;
+            if (!__any_sync(FULL, cnt > 0)) continue;
+        }
+        if (cnt > 0 && g0 + lane != mid)
+            entry_delta(a, vol, a.nbr_cell[g0 + lane], a.nbr_shift[g0 + lane], cx, cy, cz, org_i, Dx, Dy, Dz);
         int pk = 0, poff = 0;  // producer cursor
         int ck = 0, coff = 0;  // consumer cursor
         for (int s = 0; s < STAGES; ++s)

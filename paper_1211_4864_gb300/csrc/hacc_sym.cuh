@@ -37,8 +37,9 @@ __device__ __forceinline__ void entry_delta(const KArgs &a, const hacc_volume &v
 
 // Lane's entry of a group (first record jb, cnt of them) clipped to the
 // segment's j records of the task's flattened list.  before: the records of
-// the groups before, brought up to date.  size: the task's particles.
-__device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, int size, int &before, int &jb, int &cnt)
+// the groups before, brought up to date.  size: the task's particles.  False
+// once the segment has ended.
+__device__ __forceinline__ bool clip_entry(const KArgs &a, int lane, int code, int size, int &before, int &jb, int &cnt)
 {
     int inc = cnt;
 #pragma unroll
@@ -52,6 +53,7 @@ __device__ __forceinline__ void clip_entry(const KArgs &a, int lane, int code, i
     const int lo = max(first, jlo), hi = code >> 24 ? first + cnt : min(first + cnt, jlo + per);
     jb += lo - first;
     cnt = max(hi - lo, 0);
+    return code >> 24 || __shfl_sync(FULL, first, 0) < jlo + per;
 }
 
 // Without dense tasks (n_dense given and 0) the hit kernel stores every

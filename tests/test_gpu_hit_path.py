@@ -222,3 +222,36 @@ def test_segments_of_long_lists_and_full_cells(field, masses):
         rms, mx = err_norms(got.cpu().numpy().T[t].astype(np.float64), ref)
         assert rms < RMS_TOL and mx < MAX_TOL, (name, rms, mx)
     assert np.linalg.norm(gm.cpu().numpy()[t] - GM) < RMS_TOL * np.linalg.norm(GM)
+
+
+@pytest.mark.parametrize("leaf", [8, 64])
+def test_segments_of_tree_lists(leaf):
+    """Tree leaves about a blob of 6,000 particles: long lists whose length is estimated from sixteen entries, tasks cut
+    into segments, the segments' walks starting and ending inside the list."""
+    torch = need_cuda()
+    import paper_1211_4864_gb300 as hs
+    hs.load()
+    rng = np.random.default_rng(leaf)
+    pos = np.concatenate([rng.uniform(0, 18.0, (6001, 3)), 9.0 + rng.normal(size=(6000, 3))]).astype(np.float32)
+    N, L = len(pos), 18.0
+    m = rng.uniform(0.5, 2.0, N).astype(np.float32)
+    lam = rng.normal(size=(N, 3)).astype(np.float32)
+    c = default_coeffs(RC, EPS)
+    prm = hs.SRParams(EPS, RC, c)
+    sr = hs.ShortRange(L, np.array([0, N]), RC, builder="rcb", leaf_max=leaf, split_T=leaf)
+    sr.prepare(torch.tensor(pos.T.copy(), device="cuda"), torch.tensor(m, device="cuda"))
+    lt = torch.tensor(lam.T.copy(), device="cuda")
+    a = sr.force_symmetric(prm)
+    g, gm = sr.adjoint_symmetric(prm, lt)
+    torch.cuda.synchronize()
+    sr.check_status()
+    longest = (sr.nbr_off[1 : sr.n_cells + 1] - sr.nbr_off[: sr.n_cells]).max().item()
+    assert longest > 128
+    t = rng.choice(N, 800, replace=False)
+    c64 = c.astype(np.float64)
+    A = oracle.sr_force(*pos.T.copy(), m, L, EPS, RC, c64, targets=t)
+    G, GM = oracle.sr_force_adjoint(*pos.T.copy(), m, L, EPS, RC, c64, lam.astype(np.float64), targets=t)
+    for name, got, ref in (("force", a, A), ("adjoint", g, G)):
+        rms, mx = err_norms(got.cpu().numpy().T[t].astype(np.float64), ref)
+        assert rms < RMS_TOL and mx < MAX_TOL, (name, rms, mx)
+    assert np.linalg.norm(gm.cpu().numpy()[t] - GM) < RMS_TOL * np.linalg.norm(GM)
