@@ -68,6 +68,13 @@ def cached_split(config: str, default: int = 64, path: str = CACHE) -> int:
     return int(ent.get("split_T", default)) if ent else default
 
 
+def _best(ok):
+    """The fastest shape; among those within 2 % of it (every shape, where small cells leave the tuned kernel
+    little to do) the one with the most warps on an SM, which stands up best when the cells grow."""
+    least = min(t[1] for t in ok)
+    return max((t for t in ok if t[1] <= 1.02 * least), key=lambda t: (t[0].warps_per_cta * t[0].ctas_per_sm, -t[1]))
+
+
 def tune(run, config: str, mode: str = "force", quick: bool = False, reps: int = 3, path: str = CACHE,
          write: bool = True, extra: dict | None = None, cands=None):
     """Time ``run(launch)`` for every candidate; returns (best Launch, table)."""
@@ -90,7 +97,7 @@ def tune(run, config: str, mode: str = "force", quick: bool = False, reps: int =
             ts.append(e0.elapsed_time(e1))
         table.append((L, statistics.median(ts), None))
     ok = [t for t in table if t[1] is not None]
-    best = min(ok, key=lambda t: t[1])
+    best = _best(ok)
     if write:
         cache = load_cache(path)
         ent = cache.setdefault(_key(config), {})
