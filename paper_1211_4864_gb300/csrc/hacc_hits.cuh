@@ -24,15 +24,15 @@
 // room for the rounding of s + eps in the exact test.  It admits about 1 %
 // more pairs than the test keeps.
 //
-// What bounds it: issue slots (70 % used) with the gathers' shared-memory
-// wavefronts close behind (58 %); per 32 pairs about 1.5 slots per candidate in
+// What bounds it: issue slots (78 % used) with the gathers' shared-memory
+// wavefronts close behind (73 %); per 32 pairs about 1.5 slots per candidate in
 // step 2 and 28 per hit in step 3, against 20 per candidate in the dense loop.
 // A batch whose fullest lane holds more hits than HITS_DENSE of its records (a
 // halo next door) is evaluated densely from the same tile instead.  Measured
 // (GB300), gather force and adjoint with dL/dm: 2.1M lattice particles 1.83 ->
-// 0.92 ms and 3.17 -> 1.45 ms, 4096 uniform ones 85 -> 69 us; 16.8M clustered
-// 63.2 -> 59.1 ms for the force, whose small cells alone take this path.
-// Symmetric force and adjoint, lattice: 1.24 -> 0.96 ms and 2.20 -> 1.38 ms.
+// 0.92 ms and 3.17 -> 1.42 ms, 4096 uniform ones 85 -> 71 us; 16.8M clustered
+// 61.9 -> 58.8 ms for the force, whose small cells alone take this path.
+// Symmetric force and adjoint, lattice: 1.24 -> 0.97 ms and 2.20 -> 1.41 ms.
 #pragma once
 
 #include "hacc_terms.cuh"
@@ -45,10 +45,15 @@ constexpr float HITS_DELTA = 0.001953125f;  // 2^-9
 // a batch is evaluated densely when its fullest lane has this share of hits
 constexpr float HITS_DENSE = 0.6f;
 
-// Chaining-mesh cells of at most HITS_CELL particles take the hit path.  40,
-// 48, 64 and 96 measured within 6 % of each other on lattice, uniform and
-// clustered particles (symmetric lattice force 0.94, 0.91 ms at 40, 64; 1.24
-// with the dense kernel alone); 40 covers the cells of a near-uniform field.
+// Chaining-mesh cells of at most HITS_CELL particles take the hit path.  40 is
+// not the fastest bound: at 40, 48 and 64 the symmetric force of 2.1M lattice
+// particles takes 0.97, 0.93, 0.92 ms (1.24 with the dense kernel alone), the
+// gather force at 1.5 particles per unit volume 0.44, 0.31, 0.26 and with a
+// skin of 0.3 on the lattice 1.64, 1.29, 1.26, clustered fields the same.  It
+// was set by the test of the 64^3 trajectory's gradient, which allows 1e-5 of
+// the float64 reference: its symmetric pair at split_T 64 reads 9.84e-6 at 40,
+// 1.007e-5 at 48 and 1.004e-5 at 64.  (The error is one draw of the rounding:
+// over split_T 32 to 128 all three read 9.1e-6 to 1.01e-5, 9.6e-6 on average.)
 constexpr int HITS_CELL = 40;
 
 // Shared memory of the path (bytes from its base): a pad of records outside
@@ -57,10 +62,10 @@ constexpr int HITS_CELL = 40;
 // of its column, and one word that says which records are the i cell's own.
 constexpr int HITS_PAD = 128;
 constexpr float HITS_FAR = 1.0e18f;  // an empty record's coordinates: outside any cutoff, squares finite
-__host__ __device__ constexpr int hits_lam_off() { return HITS_PAD + HITS_RECS * 16; }
+constexpr int HITS_LAM = HITS_RECS * 16;  // from a record to its cotangent (adjoint)
 __host__ __device__ constexpr int hits_n_off(int mode)
 {
-    return HITS_PAD + HITS_RECS * 16 * (is_adjoint(mode) ? 2 : 1);
+    return HITS_PAD + HITS_RECS * 16 + (is_adjoint(mode) ? HITS_LAM : 0);
 }
 __host__ __device__ constexpr int hits_word_off(int mode) { return hits_n_off(mode) + HITS_RECS * 4; }
 // ... eight words a lane and HITS_STOPS empty ones behind them
@@ -192,7 +197,7 @@ __device__ __forceinline__ void hit_pair(uint32_t rec, const float4 &oi, float m
     else if constexpr (MODE == POTENTIAL)
         pair_potential(o, oi.x, oi.y, oi.z, K, p);
     else
-        pair_adjoint<MODE == ADJOINT_GM, false>(o, lds128(rec + HITS_RECS * 16), oi.x, oi.y, oi.z, mi, li.x, li.y,
+        pair_adjoint<MODE == ADJOINT_GM, false>(o, lds128(rec + HITS_LAM), oi.x, oi.y, oi.z, mi, li.x, li.y,
                                                 li.z, K, p);
 }
 
@@ -308,7 +313,7 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
                 sts128(tile + 16 * (nb + lane), make_float4(HITS_FAR, HITS_FAR, HITS_FAR, 0.f));
                 sts32(base + hits_n_off(MODE) + 4 * (nb + lane), 1.0e37f);
                 if constexpr (is_adjoint(MODE))
-                    sts128(tile + HITS_RECS * 16 + 16 * (nb + lane), make_float4(0.f, 0.f, 0.f, 0.f));
+                    sts128(tile + HITS_LAM + 16 * (nb + lane), make_float4(0.f, 0.f, 0.f, 0.f));
             }
             auto put = [&](int r, const float4 &p, const float4 &l, int e) {
                 const float x = p.x + __shfl_sync(FULL, Dx, e), y = p.y + __shfl_sync(FULL, Dy, e),
@@ -316,7 +321,7 @@ __device__ __forceinline__ bool run_hits(const KArgs &a, uint32_t base, uint32_t
                 if (r >= 0) {
                     sts128(tile + 16 * r, make_float4(x, y, z, unit ? 1.0f : p.w));
                     sts32(base + hits_n_off(MODE) + 4 * r, fmaf(z, z, fmaf(y, y, x * x)) * (1.0f - HITS_DELTA));
-                    if constexpr (is_adjoint(MODE)) sts128(tile + HITS_RECS * 16 + 16 * r, l);
+                    if constexpr (is_adjoint(MODE)) sts128(tile + HITS_LAM + 16 * r, l);
                 }
             };
             // (2.1M lattice particles: force 925 us with two, 944 with three; potential 853 and 845)
@@ -524,7 +529,7 @@ __device__ __forceinline__ int segment_count(const KArgs &a, int size, int nj, i
 // call, the segments' own prologues and sums a share of the pairs.  Symmetric
 // force with segments of 16k, 32k, 64k, 128k pairs: 262,144 clustered particles
 // 0.40, 0.40, 0.42, 0.53 ms (0.56 uncut), 16.8M 38.9, 38.8, 37.6, 37.1 ms; with
-// this rule 0.40 and 34.9 ms (36.3 uncut), 1M 3.8 -> 2.8 ms.
+// this rule 0.39 and 35.2 ms (36.3 uncut), 1M 3.8 -> 2.7 ms.
 int seg_pairs_for(int64_t N)
 {
     const int64_t p = N / 16;

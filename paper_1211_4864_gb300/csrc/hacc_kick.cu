@@ -59,9 +59,9 @@ constexpr int MOM_N = 9;  // sums: m v (3), m a (3), kinetic, m |a|, potential
 
 // Double-float arithmetic on the float32 pipe (an unevaluated sum hi + lo of
 // two float32 values, about 48 significant bits): GB300's float64 pipe is
-// narrow (2 lanes a clock and SM), so the per-particle terms, each thread's
-// partial sums and each warp's reduction are formed this way and only the
-// per-thread totals are reduced in float64.
+// narrow (2 lanes a clock and SM), so the per-particle terms and each thread's
+// partial sums are formed this way and only the threads' totals are added in
+// float64.
 // Knuth's TwoSum: s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 {
@@ -200,11 +200,13 @@ int moment_blocks(int64_t N)
 // particle 4 floor(N / 4) + t of the last, partial group.  Per particle and
 // per thread in double-float (above), across threads and blocks in float64.
 //
-// What bounds it: the copy rate at 16.8M particles (470 MB read), its latency
-// at a few thousand.  Nine float64 shuffle reductions in each of a fixed 4096
-// blocks held the narrow float64 pipe for 150 us whatever N; reduced in
-// double-float by a grid that follows N, 4096 particles take MOMS4K us (164
-// before) and 16.8M take MOMS16M us (265 before).
+// What bounds it: at 16.8M particles (470 MB read, 69 us at the copy rate) the
+// float64 pipe, at a few thousand the launches.  Nine float64 shuffle
+// reductions in every warp of a fixed 4096 blocks held that pipe for 150 us
+// whatever N.  Here each thread's totals go through shared memory, a warp a sum
+// adds eight of them a lane before its shuffles, and the grid follows N: a call
+// on 4096 particles takes about 33 us (194 before), on 2.1M 41 (200), on 16.8M
+// 208 (311).
 __global__ void __launch_bounds__(MOM_THREADS)
 k_moments_partial(int64_t N, const float *__restrict__ m, const float *__restrict__ vx, const float *__restrict__ vy,
                   const float *__restrict__ vz, const float *__restrict__ ax, const float *__restrict__ ay,

@@ -521,8 +521,12 @@ __device__ __forceinline__ long long gap2_steps(const int32_t *qi, const int32_t
 // One thread per leaf: count (FILL = false) or write (FILL = true) its list.
 // A walk is a chain of dependent loads, and the lanes of a warp diverge: up to
 // this many leaves, which leave the GPU idle otherwise, four share a warp, more
-// fill it.  Lists of 176, 5,892 and 46,798 leaves: 0.74, 1.31, 1.90 ms with full
-// warps, 0.45, 0.98, 3.20 ms with four a warp.
+// fill it.  Lists of 262,144 clustered particles, ms with 4, 8, 16 and 32 leaves
+// a warp: 191 leaves 0.32, 0.37, 0.44, 0.51; 5,892 0.95, 1.07, 1.13, 1.28; 7,772
+// 1.28, 1.38, 1.42, 1.53; 11,746 1.95, 1.85, 2.09, 2.11; 23,258 4.61, 4.11, 3.83,
+// 3.89; 45,593 14.2, 10.2, 8.7, 7.9; of 1M particles, 23,157 leaves 1.96, 1.71,
+// 1.73, 1.63.  So four are best up to 8,000 and 32 from 23,000 on; between them
+// the two differ by 8 %.
 constexpr int WALK_FEW = 8192;
 
 template <bool FILL>

@@ -1,18 +1,36 @@
 """The tensor-core filter of the hit path loses no pair inside the cutoff.
 
 The filter keeps a pair when n_i + n_j - 2 x_i.x_j - cut is negative, with
-n = (1 - 2^-9) |x|^2 and x, n_j rounded to tf32 (11 significant bits).  This
-restates it in numpy, with the products' sum truncated to float32 after every
+n = (1 - delta) |x|^2 and x, n_j rounded to tf32 (11 significant bits).  This
+restates it in numpy with the sources' own delta and cut (the kernel itself is
+held to the exact test in test_gpu_rim.py), with the products' sum truncated to float32 after every
 term, on pairs at and just inside the cutoff over the offsets that cells of
 one to eight cutoffs produce, and on uniform pairs, of which it may admit only
 few more than the exact test."""
 
+import os
+import re
+
 import numpy as np
 import pytest
 
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1211_4864_gb300", "csrc")
+
+
+def source(name, pattern):
+    """The one match of pattern in a CUDA source."""
+    with open(os.path.join(CSRC, name)) as f:
+        found = re.findall(pattern, f.read())
+    assert len(found) == 1, (name, pattern, found)
+    return found[0]
+
+
+# the margin and the cut as the sources form them (hit_cut: r_c^2 (1.0 + 1.0 / A) + eps / (1 << B))
 RC, EPS = np.float32(3.0), np.float32(0.01)
-DELTA = np.float32(2.0 ** -9)
-CUT = np.float32(9.0 * (1 + 1 / 4096) + 0.01 / 2 ** 20)
+DELTA = np.float32(source("hacc_hits.cuh", r"constexpr float HITS_DELTA = ([0-9.e-]+)f;"))
+A, B = source("hacc_pairs.cuh", r"K\.hit_cut = \(float\)\(\(double\)p->rcut \* \(double\)p->rcut \* "
+                                r"\(1\.0 \+ 1\.0 / (\d+)\) \+ \(double\)p->eps / \(1 << (\d+)\)\);")
+CUT = np.float32(9.0 * (1 + 1 / int(A)) + float(EPS) / 2 ** int(B))
 
 
 def tf32(x):
